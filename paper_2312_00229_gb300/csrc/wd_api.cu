@@ -383,6 +383,8 @@ int weno_zoom2x_bwd(const weno_image* x, const weno_image* grad_out, const weno_
   a.gi_sc = grad_in->stride_c; a.gi_sh = grad_in->stride_h; a.gi_sw = grad_in->stride_w;
   a.orows = orows;
   a.ocols = ocols;
+  a.g_vec = a.g_sw == 1 && a.g_sh % 2 == 0 && a.g_sc % 2 == 0 &&
+            reinterpret_cast<uintptr_t>(a.gout) % 8 == 0;
   a.ws = static_cast<float*>(workspace);
   cudaError_t e = launch_zoom2x_bwd(a, k, bmode, static_cast<cudaStream_t>(stream));
   return e == cudaSuccess ? WENO_OK : WENO_ECUDA;

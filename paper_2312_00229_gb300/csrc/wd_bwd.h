@@ -20,6 +20,7 @@ struct BwdArgs {
   int64_t g_sc, g_sh, g_sw;
   int64_t gi_sc, gi_sh, gi_sw;
   int64_t orows, ocols;
+  int g_vec;  // output-gradient columns 2c, 2c + 1 load as one aligned float2
   float* ws;  // 2 * (n + 2 BWD_GHOST) * (m + 2 BWD_GHOST) * planes floats
 };
 
