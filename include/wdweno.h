@@ -146,8 +146,9 @@ size_t weno_zoom2x_batched_workspace_bytes(int count);
  *                 the call can be captured into a CUDA graph and replayed)
  *   workspace   : device buffer of >= weno_zoom2x_batched_workspace_bytes
  *                 bytes; contents need no initialisation and are scratch
- *   rows_per_tile, tile_width : tile shape (0 = library default: 128-row
- *                 bands, 247-column strips); tile_width takes the values of
+ *   rows_per_tile, tile_width : tile shape (0 = library default: a band
+ *                 height chosen on the device from the images' sizes,
+ *                 118-column strips); tile_width takes the values of
  *                 weno_zoom2x_fwd_tiled (247, 119, 246, 118); narrower
  *                 strips leave a smaller part of each image's last strip
  *                 idle, which pays for narrow images; the autotuner chooses
@@ -163,16 +164,14 @@ int weno_zoom2x_batched(int count, const weno_image* d_in, weno_dtype in_t,
 
 /* weno_zoom2x_fwd with an explicit tile shape, for the autotuner.
  *   rows_per_tile : coarse rows per CTA band, 1..4096 (0 = the default:
- *                   the band count that best balances the last wave of CTAs
- *                   on this GPU against the per-band pipeline fill)
+ *                   the band height, and with tile_width 0 the width, of
+ *                   least modelled time on this GPU)
  *   tile_width    : coarse output columns per CTA, which also fixes the
  *                   coarse columns each thread owns: 247 (256 threads of one
  *                   column, 9 columns covering the dependency halo), 119
  *                   (128 threads of one column), 246 (128 threads of two
  *                   adjacent columns, 10 halo columns), 118 (64 threads of
- *                   two), or 0 = the library's choice for the image width
- *                   (the shape that spends the fewest column-steps across
- *                   it).  Every shape gives bit-identical outputs.
+ *                   two), or 0 = the library's choice.  Every shape gives bit-identical outputs.
  * Returns as weno_zoom2x_fwd, or WENO_EINVAL for an unsupported shape and
  * WENO_ERANGE when the band count exceeds 65535. */
 int weno_zoom2x_fwd_tiled(const weno_image* in, weno_dtype in_t, const weno_image* out,

@@ -18,13 +18,6 @@ using namespace wdweno;
 
 namespace {
 
-constexpr int64_t kDefaultRowsPerBand = 64;
-// Persistent batched launches: 128-row bands measured best on 256 FP16 images
-// of sides 64..1024 (77.2 Gpix/s at 64 rows, 78.7 at 128, 76.7 at 192); the
-// queue still holds some 10,000 tiles for 304 CTA slots.
-constexpr int64_t kBatchedRowsPerBand = 128;
-constexpr int kFwdCtasPerSm = 2;  // 256-thread CTAs x 128 registers (twice as many at 128)
-
 int sm_count() {
   static int cached[64] = {0};
   int dev = 0;
@@ -49,35 +42,6 @@ bool shape_for_width(int tile_width, int* threads, int* cols) {
   if (tile_width == 2 * 128 - 10) { *threads = 128; return true; }
   if (tile_width == 2 * 64 - 10) { *threads = 64; return true; }
   return false;
-}
-
-// Band height for a one-launch forward: choose the number of bands B that
-// minimises (waves of CTAs) x (rows per band + pipeline fill), i.e. balance
-// the tail of the last wave against the fixed per-band cost.  `cols` coarse
-// columns per thread: one-column CTAs of 256 (128) threads keep 2 (4)
-// resident per SM, two-column CTAs of 128 (64) threads 3 (6).
-int64_t default_rows_per_band(int64_t n, int64_t m, int64_t planes, int threads, int cols = 1) {
-  const int sms = sm_count();
-  if (sms <= 0) return kDefaultRowsPerBand;
-  const int64_t per_sm = cols == 2 ? 3 * 128 / threads : kFwdCtasPerSm * (threads_fwd() / threads);
-  const int64_t slots = (int64_t)sms * per_sm;
-  const int64_t tw = cols == 2 ? 2 * threads - 10 : threads - 9;
-  const int64_t strips = (m + tw - 1) / tw;
-  const int64_t base = strips * planes;
-  const int64_t fill = 7;  // extra steps per band: 4 + 5 halo rows + 2 pipeline steps
-  int64_t best_rpb = n, best_cost = -1;
-  for (int64_t bands = 1; bands <= 4096; ++bands) {
-    const int64_t rpb = (n + bands - 1) / bands;
-    if (rpb < 16 && bands > 1) break;
-    if (bands > 1 && (n + rpb - 1) / rpb != bands) continue;  // same rpb as a smaller count
-    const int64_t waves = (base * bands + slots - 1) / slots;
-    const int64_t cost = waves * (rpb + fill);
-    if (best_cost < 0 || cost < best_cost) {
-      best_cost = cost;
-      best_rpb = rpb;
-    }
-  }
-  return best_rpb < 1 ? 1 : best_rpb;
 }
 
 int64_t dtype_size(int dt) {
@@ -230,12 +194,7 @@ FwdArgs make_fwd_args(const weno_image* in, int in_t, const weno_image* out, int
   a.orows = orows;
   a.ocols = ocols;
   a.rows_per_band = rows_per_band;
-  const int64_t esz = dtype_size(out_t);
-  const uintptr_t base = reinterpret_cast<uintptr_t>(out->data);
-  a.out_vec = (out->stride_w == 1) && (out->stride_h % 2 == 0) && (out->stride_c % 2 == 0) &&
-              (base % uintptr_t(2 * esz) == 0);
-  a.out_vec4 = (out->stride_w == 1) && (out->stride_h % 4 == 0) && (out->stride_c % 4 == 0) &&
-               (base % uintptr_t(4 * esz) == 0);
+  set_store_modes(a, dtype_size(out_t));
   a.cols = 1;
   return a;
 }
@@ -269,7 +228,7 @@ bool cascade_plan(const weno_image* in, int levels, const weno_params& p, Cascad
     if (c->n[L + 1] < 1 || c->m[L + 1] < 1 || c->n[L + 1] >= (int64_t(1) << 31) ||
         c->m[L + 1] >= (int64_t(1) << 31))
       return false;
-    c->rpb[L] = default_rows_per_band(c->n[L], c->m[L], in->channels, CASCADE_THREADS);
+    c->rpb[L] = fwd_plan_for(c->n[L], c->m[L], in->channels, sm_count(), CASCADE_THREADS, 1, 0).rows;
   }
   c->done_count = 0;
   for (int L = 0; L < levels; ++L) {
@@ -322,21 +281,17 @@ int weno_zoom2x_fwd_tiled(const weno_image* in, weno_dtype in_t, const weno_imag
   if (rc != WENO_OK) return rc;
   if (rows_per_tile < 0 || rows_per_tile > 4096) return WENO_EINVAL;
   int threads = 0, cols = 1;
-  if (tile_width == 0) {
-    fwd_shape_for(in->width, &threads, &cols);
-  } else if (!shape_for_width(tile_width, &threads, &cols)) {
-    return WENO_EINVAL;
-  }
+  if (tile_width != 0 && !shape_for_width(tile_width, &threads, &cols)) return WENO_EINVAL;
   MethodConsts k;
   int bmode;
   if (!fold_consts(p, &k, &bmode)) return WENO_EINVAL;
-  const int64_t rpb = rows_per_tile > 0 ? rows_per_tile
-                                        : default_rows_per_band(in->height, in->width,
-                                                                in->channels, threads, cols);
+  const FwdPlan plan = fwd_plan_for(in->height, in->width, in->channels, sm_count(), threads, cols,
+                                    rows_per_tile);
+  const int64_t rpb = plan.rows;
   if (bmode == B2 && direct_b2_ok(p, in_t)) bmode = B2R;
   FwdArgs a = make_fwd_args(in, in_t, out, out_t, orows, ocols, rpb);
-  a.threads = threads;
-  a.cols = cols;
+  a.threads = plan.threads;
+  a.cols = plan.cols;
   if ((a.n + rpb - 1) / rpb > 65535) return WENO_ERANGE;
   cudaError_t e = launch_zoom2x_fwd(a, k, bmode, static_cast<cudaStream_t>(stream));
   return e == cudaSuccess ? WENO_OK : WENO_ECUDA;
@@ -408,7 +363,7 @@ int weno_zoom2x_batched(int count, const weno_image* d_in, weno_dtype in_t,
   if (!workspace || workspace_bytes < batched_workspace_bytes(count)) return WENO_EWORKSPACE;
   if (reinterpret_cast<uintptr_t>(workspace) % 16 != 0) return WENO_EWORKSPACE;
   if (rows_per_tile < 0 || rows_per_tile > 4096) return WENO_EINVAL;
-  int threads = threads_fwd(), cols = 1;
+  int threads = 64, cols = 2;  // the best or within 5% of it from 5 small to 256 large images
   if (tile_width != 0 && !shape_for_width(tile_width, &threads, &cols)) return WENO_EINVAL;
   MethodConsts k;
   int bmode;
@@ -423,7 +378,8 @@ int weno_zoom2x_batched(int count, const weno_image* d_in, weno_dtype in_t,
   a.in_dtype = in_t;
   a.out_dtype = out_t;
   a.out_mode = p.out_mode;
-  a.rows_per_band = rows_per_tile > 0 ? rows_per_tile : kBatchedRowsPerBand;
+  a.rows_per_band = rows_per_tile;  // 0: chosen on the device from the images' sizes
+  a.sms = sm_count();
   a.workspace = workspace;
   cudaError_t e = launch_zoom2x_batched(a, k, bmode, static_cast<cudaStream_t>(stream));
   return e == cudaSuccess ? WENO_OK : WENO_ECUDA;

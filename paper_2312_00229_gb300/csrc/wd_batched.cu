@@ -3,7 +3,8 @@
 //
 // Workspace (caller-owned, no initialisation needed):
 //   [0]   unsigned long long  head, next tile
-//   [8]   unsigned long long  total, tiles of all images
+//   [8]   unsigned long long  total, tiles of all images; rows per band in the
+//                             top 16 bits
 //   [16]  unsigned long long  prefix[count + 1], the exclusive prefix sum of
 //                             the tiles of each image (a malformed image has
 //                             none)
@@ -12,6 +13,7 @@
 // persistent kernel is in wd_batched_kernel.cuh; this unit instantiates it
 // with one coarse column per thread, wd_batched2.cu with two.
 #include "wd_batched_kernel.cuh"
+#include "wd_fwd_model.h"
 
 namespace wdweno {
 
@@ -36,46 +38,152 @@ __device__ bool descriptor_ok(const weno_image& in, const weno_image& out, int o
          out.channels == in.channels;
 }
 
-// Tiles of one image for CTAs of `threads` x `cols` columns.
-__device__ unsigned long long image_tiles(const weno_image& in, int64_t rpb, int threads,
-                                          int cols) {
-  const unsigned long long tw = (unsigned long long)strip_width(threads, cols);
-  const unsigned long long strips = (in.width + tw - 1) / tw;
-  const unsigned long long bands = (in.height + rpb - 1) / rpb;
+// Tiles of one image with bands of at most `rows` rows and strips of `tw`
+// columns.
+__device__ unsigned long long image_tiles(const weno_image& in, int64_t rows, int tw) {
+  const unsigned long long strips = ((unsigned long long)in.width + tw - 1) / tw;
+  const int64_t r = batched::even_band(in.height, rows);
+  const unsigned long long bands = (unsigned long long)((in.height + r - 1) / r);
   return strips * bands * (unsigned long long)in.channels;
 }
 
-__global__ void __launch_bounds__(SETUP_THREADS) batched_setup_kernel(BatchedArgs a) {
+// Band heights the setup kernel chooses from.
+constexpr int CANDS = 13;
+__constant__ int g_cands[CANDS] = {3, 4, 6, 8, 12, 16, 24, 32, 48, 64, 96, 128, 192};
+// A tile's steps beyond its rows (the fill, the ring clearing, the ticket and
+// the descriptor), and the part of the longest tile that the end of the queue
+// costs.  With these the choice was the best of the measured heights (4 .. 192)
+// on each of the five batches below; 16 to 18 and 0.2 to 0.3 choose the same.
+constexpr float TILE_FILL = 17.f;
+constexpr float TILE_TAIL = 0.25f;
+
+// What a band height would cost, summed over a thread's images.
+struct Cost {
+  float tiles, steps, longest;
+};
+
+__device__ __forceinline__ float warp_sum(float v) {
+  for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+__device__ __forceinline__ float warp_max(float v) {
+  for (int o = 16; o; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+  return v;
+}
+
+// One CTA: validates the descriptors, chooses the band height where the
+// caller left it open, and writes the exclusive prefix sum of tiles.
+//
+// The choice takes the band height with the least modelled time: the steps of
+// all tiles shared by the resident CTAs, plus a part of a tile for the end of
+// the queue, but never less than the longest tile; a step's time follows
+// wd_fwd_model.h.  Before, the default was 128 rows and one-column strips of
+// 247, which leaves small batches on a few CTAs: 5 uint8 images of sides
+// 48..96, 102 us (17 us with the choice); 16 of 100..400, 111 us (56); 30 BF16 planes
+// of 64..512, 116 us (60); 64 FP16 images of 64..1024, 852 us (675); 256 uint8, 2986
+// us (2294).
+__global__ void __launch_bounds__(SETUP_THREADS) batched_setup_kernel(BatchedArgs a,
+                                                                      FwdShape shape) {
   Queue* q = static_cast<Queue*>(a.workspace);
-  __shared__ unsigned long long part[SETUP_THREADS];
-  const int t = threadIdx.x;
+  __shared__ unsigned long long part[SETUP_THREADS / 32];
+  __shared__ float c_tiles[CANDS], c_steps[CANDS];
+  __shared__ int c_longest[CANDS];
+  __shared__ int s_rows;
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const int tw = strip_width(a.threads, a.cols);
   const int chunk = (a.count + SETUP_THREADS - 1) / SETUP_THREADS;
   const int lo = min(a.count, t * chunk), hi = min(a.count, lo + chunk);
+  int64_t rows = a.rows_per_band;
+  if (rows <= 0) {
+    if (t < CANDS) {
+      c_tiles[t] = c_steps[t] = 0.f;
+      c_longest[t] = 0;
+    }
+    __syncthreads();
+    Cost c[CANDS];
+#pragma unroll
+    for (int j = 0; j < CANDS; ++j) c[j] = Cost{0.f, 0.f, 0.f};
+    for (int i = lo; i < hi; ++i) {
+      const weno_image in = a.in[i], out = a.out[i];
+      if (!descriptor_ok(in, out, a.out_mode)) continue;
+      const float strips = float((in.width + tw - 1) / tw) * float(in.channels);
+      const int n = (int)in.height;
+#pragma unroll
+      for (int j = 0; j < CANDS; ++j) {
+        const int r0 = g_cands[j], b0 = (n - 1) / r0 + 1, r = (n - 1) / b0 + 1;
+        const float bands = float((n - 1) / r + 1);
+        c[j].tiles += strips * bands;
+        c[j].steps += strips * (float(n) + bands * TILE_FILL);
+        c[j].longest = fmaxf(c[j].longest, float(r));
+      }
+    }
+    if (warp * 32 * chunk < a.count) {  // warps with images
+#pragma unroll
+      for (int j = 0; j < CANDS; ++j) {
+        const float tiles = warp_sum(c[j].tiles), steps = warp_sum(c[j].steps);
+        const float longest = warp_max(c[j].longest);
+        if (lane == 0) {
+          atomicAdd(&c_tiles[j], tiles);
+          atomicAdd(&c_steps[j], steps);
+          atomicMax(&c_longest[j], (int)longest);
+        }
+      }
+    }
+    __syncthreads();
+    if (warp == 0) {
+      float us = 3.0e38f;
+      if (lane < CANDS && c_tiles[lane] > 0.f) {
+        const float k = fminf(float(shape.per_sm), ceilf(c_tiles[lane] / float(a.sms)));
+        const float one = float(c_longest[lane]) + TILE_FILL;
+        const float steps = fmaxf(one, c_steps[lane] / (float(a.sms) * k) + TILE_TAIL * one);
+        us = steps * sqrtf(shape.lat * shape.lat + k * k * shape.issue * shape.issue);
+      }
+      int best = lane;
+      for (int o = 16; o; o >>= 1) {
+        const float v = __shfl_xor_sync(0xffffffffu, us, o);
+        const int w = __shfl_xor_sync(0xffffffffu, best, o);
+        if (v < us || (v == us && w < best)) {
+          us = v;
+          best = w;
+        }
+      }
+      if (lane == 0) s_rows = g_cands[best < CANDS ? best : 0];
+    }
+    __syncthreads();
+    rows = s_rows;
+  }
   unsigned long long sum = 0ULL;
   for (int i = lo; i < hi; ++i) {
     const weno_image in = a.in[i], out = a.out[i];
-    if (descriptor_ok(in, out, a.out_mode))
-      sum += image_tiles(in, a.rows_per_band, a.threads, a.cols);
+    if (descriptor_ok(in, out, a.out_mode)) sum += image_tiles(in, rows, tw);
   }
-  part[t] = sum;
+  // inclusive scan over the threads: within warps, then over their totals
+  unsigned long long scan = sum;
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned long long v = __shfl_up_sync(0xffffffffu, scan, o);
+    if (lane >= o) scan += v;
+  }
+  if (lane == 31) part[warp] = scan;
   __syncthreads();
-  // Inclusive Hillis-Steele scan of the per-thread sums.
-  for (int off = 1; off < SETUP_THREADS; off <<= 1) {
-    const unsigned long long v = t >= off ? part[t - off] : 0ULL;
-    __syncthreads();
-    part[t] += v;
-    __syncthreads();
+  if (warp == 0) {
+    unsigned long long v = part[lane];
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned long long u = __shfl_up_sync(0xffffffffu, v, o);
+      if (lane >= o) v += u;
+    }
+    part[lane] = v;
   }
-  unsigned long long run = part[t] - sum;  // exclusive start
+  __syncthreads();
+  if (warp > 0) scan += part[warp - 1];
+  unsigned long long run = scan - sum;  // exclusive start
   for (int i = lo; i < hi; ++i) {
     q->prefix[i] = run;
     const weno_image in = a.in[i], out = a.out[i];
-    if (descriptor_ok(in, out, a.out_mode))
-      run += image_tiles(in, a.rows_per_band, a.threads, a.cols);
+    if (descriptor_ok(in, out, a.out_mode)) run += image_tiles(in, rows, tw);
   }
   if (t == SETUP_THREADS - 1) {
-    q->prefix[a.count] = part[t];
-    q->total = part[t];
+    q->prefix[a.count] = scan;
+    q->total = scan | ((unsigned long long)rows << batched::ROWS_SHIFT);
     q->head = 0ULL;
   }
 }
@@ -89,7 +197,10 @@ size_t batched_workspace_bytes(int count) {
 
 cudaError_t launch_zoom2x_batched(const BatchedArgs& a, const MethodConsts& k, int bmode,
                                   cudaStream_t stream) {
-  batched_setup_kernel<<<1, SETUP_THREADS, 0, stream>>>(a);
+  FwdShape shape = FWD_SHAPES[0];
+  for (const FwdShape& s : FWD_SHAPES)
+    if (s.threads == a.threads && s.cols == a.cols) shape = s;
+  batched_setup_kernel<<<1, SETUP_THREADS, 0, stream>>>(a, shape);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   if (a.cols == 2) return launch_batched_paired(a, k, bmode, stream);

@@ -3,6 +3,7 @@
 // per thread; wd_batched2.cu: two), which compile in parallel.
 #pragma once
 
+#include <atomic>
 #include <type_traits>
 
 #include "wd_batched.h"
@@ -14,11 +15,20 @@ namespace batched {
 using fwd_tile::THREADS;
 using fwd_tile::THREADS_NARROW;
 
+// `total`: tiles of all images in the low 48 bits, rows per band above.
 struct Queue {
   unsigned long long head;
   unsigned long long total;
   unsigned long long prefix[1];  // count + 1 entries
 };
+constexpr int ROWS_SHIFT = 48;
+
+// Rows of an image's bands: at most `rows` each, as even as the band count
+// allows (a short last band costs a whole pipeline fill).
+__device__ __forceinline__ int64_t even_band(int64_t n, int64_t rows) {
+  const int64_t bands = (n + rows - 1) / rows;
+  return (n + bands - 1) / bands;
+}
 
 __host__ __device__ __forceinline__ int64_t dsize(int dt) {
   return dt == DT_U8 ? 1 : (dt == DT_F32 ? 4 : 2);
@@ -44,30 +54,42 @@ __global__ void __launch_bounds__(NT, (BatchedShape<NT, COLS>::MIN_BLOCKS))
   __shared__ unsigned long long s_tile;
   __shared__ int s_img;
   Queue* q = static_cast<Queue*>(a.workspace);
-  const unsigned long long total = q->total;
+  const unsigned long long total = q->total & ((1ULL << ROWS_SHIFT) - 1);
+  const int64_t rows = (int64_t)(q->total >> ROWS_SHIFT);
   const unsigned long long* prefix = q->prefix;
+  // the next ticket is drawn while a tile runs, so that only the search's
+  // loads stand between two tiles
+  unsigned long long ticket = 0;
+  if (threadIdx.x == 0) ticket = atomicAdd(&q->head, 1ULL);
   for (;;) {
-    if (threadIdx.x == 0) {
-      const unsigned long long tile = atomicAdd(&q->head, 1ULL);
-      int img = -1;
+    if (threadIdx.x < 32) {
+      const int lane = threadIdx.x;
+      const unsigned long long tile = __shfl_sync(0xffffffffu, ticket, 0);
+      int lo = -1;
       if (tile < total) {
         // largest i with prefix[i] <= tile < prefix[i + 1] (images with no
-        // tiles are skipped by "largest")
-        int lo = 0, hi = a.count - 1;
-        while (lo < hi) {
-          const int mid = (lo + hi + 1) >> 1;
-          if (prefix[mid] <= tile) lo = mid; else hi = mid - 1;
+        // tiles are skipped by "largest"), 32 probes at a time
+        lo = 0;
+        int n = a.count;
+        while (n > 1) {
+          const int stride = (n + 31) / 32;
+          const bool below = lane * stride < n && __ldg(&prefix[lo + lane * stride]) <= tile;
+          const int top = 31 - __clz(__ballot_sync(0xffffffffu, below));
+          lo += top * stride;
+          n = min(stride, n - top * stride);
         }
-        img = lo;
       }
-      s_tile = tile;
-      s_img = img;
+      if (lane == 0) {
+        s_tile = tile;
+        s_img = lo;
+      }
     }
     __syncthreads();
     const int img = s_img;
     const unsigned long long tile = s_tile;
     __syncthreads();  // s_tile / s_img are rewritten only after everyone read them
     if (img < 0) break;
+    if (threadIdx.x == 0) ticket = atomicAdd(&q->head, 1ULL);
     const weno_image in = a.in[img], out = a.out[img];
     FwdArgs f;
     f.in = in.data;
@@ -81,12 +103,8 @@ __global__ void __launch_bounds__(NT, (BatchedShape<NT, COLS>::MIN_BLOCKS))
     f.out_sc = out.stride_c; f.out_sh = out.stride_h; f.out_sw = out.stride_w;
     f.orows = out.height;
     f.ocols = out.width;
-    f.rows_per_band = a.rows_per_band;
-    const uintptr_t base = reinterpret_cast<uintptr_t>(out.data);
-    f.out_vec = out.stride_w == 1 && out.stride_h % 2 == 0 && out.stride_c % 2 == 0 &&
-                base % uintptr_t(2 * dsize(a.out_dtype)) == 0;
-    f.out_vec4 = out.stride_w == 1 && out.stride_h % 4 == 0 && out.stride_c % 4 == 0 &&
-                 base % uintptr_t(4 * dsize(a.out_dtype)) == 0;
+    f.rows_per_band = even_band(f.n, rows);
+    set_store_modes(f, dsize(a.out_dtype));
     const unsigned long long local = tile - prefix[img];
     constexpr unsigned long long tw = strip_width(NT, COLS);
     const unsigned long long strips = (f.m + tw - 1) / tw;
@@ -103,18 +121,27 @@ __global__ void __launch_bounds__(NT, (BatchedShape<NT, COLS>::MIN_BLOCKS))
   }
 }
 
-inline int persistent_grid(const void* kernel, int threads) {
+// CTAs of a persistent launch: SMs x resident CTAs of the kernel (a function of
+// the device and the kernel, asked once per pair).
+template <int BMODE, class IO, int NT, int COLS>
+int persistent_grid() {
+  static std::atomic<int> known[64];
   int dev = 0, sms = 0, per_sm = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+  if (dev >= 0 && dev < 64 && known[dev].load(std::memory_order_relaxed) > 0)
+    return known[dev].load(std::memory_order_relaxed);
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, 0) != cudaSuccess)
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+          &per_sm, (const void*)batched_fwd_kernel<BMODE, IO, NT, COLS>, NT, 0) != cudaSuccess)
     return 0;
-  return sms * (per_sm > 0 ? per_sm : 1);
+  const int grid = sms * (per_sm > 0 ? per_sm : 1);
+  if (dev >= 0 && dev < 64) known[dev].store(grid, std::memory_order_relaxed);
+  return grid;
 }
 
 template <int BMODE, class IO, int NT, int COLS>
 cudaError_t launch_width(const BatchedArgs& a, const MethodConsts& k, cudaStream_t stream) {
-  const int grid = persistent_grid((const void*)batched_fwd_kernel<BMODE, IO, NT, COLS>, NT);
+  const int grid = persistent_grid<BMODE, IO, NT, COLS>();
   if (grid <= 0) return cudaErrorInvalidValue;
   batched_fwd_kernel<BMODE, IO, NT, COLS><<<grid, NT, 0, stream>>>(a, k);
   return cudaGetLastError();

@@ -2,8 +2,11 @@
 // planes, one CTA per tile.  The tile body is in wd_fwd_tile.cuh.  Storage
 // types are compile-time parameters for the common pairs (wd_fwd_typed.cu);
 // any other pair, and beta != 2, goes through the run-time-typed kernels here.
+#include <cmath>
+
 #include "wd_cascade.h"
 #include "wd_fwd_kernels.cuh"
+#include "wd_fwd_model.h"
 
 namespace wdweno {
 
@@ -13,25 +16,69 @@ cudaError_t launch_fwd_typed(const FwdArgs& a, const MethodConsts& k, int bmode,
 int tile_width_fwd() { return fwd_tile::TILE_W; }
 int threads_fwd() { return fwd_tile::THREADS; }
 
-void fwd_shape_for(int64_t m, int* threads, int* cols) {
-  // Column-steps a launch spends across the width: strips x columns per
-  // strip, a two-column column counted 0.9 of a one-column one (it issues
-  // about 16% fewer instructions per column; measured 4-9% faster on wide
-  // images).  Ties go to the earlier entry.
-  struct Shape { int threads, cols; double weight; };
-  const Shape shapes[4] = {{128, 2, 0.9}, {64, 2, 0.9}, {fwd_tile::THREADS, 1, 1.0},
-                           {fwd_tile::THREADS_NARROW, 1, 1.0}};
-  double best = 1e300;
-  for (const Shape& s : shapes) {
-    const int64_t span = (int64_t)s.threads * s.cols;  // columns of one CTA
-    const int64_t tw = s.cols == 2 ? span - 10 : span - 9;
-    const double cost = double((m + tw - 1) / tw) * double(span) * s.weight;
-    if (cost < best - 1e-9) {
-      best = cost;
-      *threads = s.threads;
-      *cols = s.cols;
+namespace {
+
+double step_us(const FwdShape& s, int64_t k) {
+  return std::sqrt(double(s.lat) * s.lat + double(k) * k * s.issue * s.issue);
+}
+
+// A plan is a function of its key alone, so the last ones are remembered (per
+// thread, a direct-mapped table): finding one scans some hundred candidates,
+// about 10 us of host time.
+struct PlanKey {
+  int64_t n, m, planes, rows;
+  int sms, threads, cols;
+  bool operator==(const PlanKey& o) const {
+    return n == o.n && m == o.m && planes == o.planes && rows == o.rows && sms == o.sms &&
+           threads == o.threads && cols == o.cols;
+  }
+};
+struct PlanSlot {
+  bool used;
+  PlanKey key;
+  FwdPlan plan;
+};
+
+FwdPlan find_plan(const PlanKey& q) {
+  FwdPlan best{fwd_tile::THREADS, 1, q.rows > 0 ? q.rows : q.n};
+  double best_us = 1e300;
+  for (const FwdShape& s : FWD_SHAPES) {
+    if (q.threads != 0 && (s.threads != q.threads || s.cols != q.cols)) continue;
+    const int64_t base = (q.m + fwd_strip(s) - 1) / fwd_strip(s) * q.planes;
+    const int64_t slots = (int64_t)q.sms * s.per_sm;
+    const double full = step_us(s, s.per_sm);
+    int64_t last = -1;
+    for (int64_t bands = 1; bands <= q.n; ++bands) {
+      const int64_t rows = q.rows > 0 ? q.rows : (q.n + bands - 1) / bands;
+      if (rows == last) continue;
+      // bands below 16 rows only where they still find idle CTA slots
+      if (bands > 1 && (rows < 2 || (rows < 16 && base * bands > 2 * slots))) break;
+      last = rows;
+      const int64_t ctas = base * ((q.n + rows - 1) / rows);
+      const int64_t rest = ctas % slots;
+      double t = double(ctas / slots) * full;
+      if (rest) t += step_us(s, (rest + q.sms - 1) / q.sms);
+      t *= double(rows < q.n ? rows : q.n) + FWD_FILL;
+      if (t < best_us - 1e-9) {
+        best_us = t;
+        best = FwdPlan{s.threads, s.cols, rows};
+      }
+      if (q.rows > 0) break;
     }
   }
+  return best;
+}
+
+}  // namespace
+
+FwdPlan fwd_plan_for(int64_t n, int64_t m, int64_t planes, int sms, int threads, int cols,
+                     int64_t rows) {
+  const PlanKey key{n, m, planes, rows, sms > 0 ? sms : 152, threads, cols};
+  static thread_local PlanSlot table[64];
+  const uint64_t h = (uint64_t)(n * 1000003 + m * 10007 + planes * 101 + rows * 7 + threads + cols);
+  PlanSlot& slot = table[(h ^ (h >> 17)) & 63];
+  if (!slot.used || !(slot.key == key)) slot = PlanSlot{true, key, find_plan(key)};
+  return slot.plan;
 }
 
 cudaError_t launch_zoom2x_fwd(const FwdArgs& a, const MethodConsts& k, int bmode,

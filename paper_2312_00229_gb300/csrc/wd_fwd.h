@@ -23,11 +23,28 @@ struct FwdArgs {
   int cols;                      // coarse columns per thread: 1, or 2 (paired tile)
 };
 
-// CTA shape of a one-launch forward over images m columns wide: `threads`
-// per CTA and `cols` coarse columns per thread (1: 256 or 128 threads, 247
-// or 119 output columns per strip; 2: 128 or 64 threads, 246 or 118), the
-// one that spends the fewest weighted column-steps across the width.
-void fwd_shape_for(int64_t m, int* threads, int* cols);
+// How output elements of `esz` bytes can be stored together.
+__host__ __device__ inline void set_store_modes(FwdArgs& a, int64_t esz) {
+  const uint64_t base = reinterpret_cast<uint64_t>(a.out);
+  a.out_vec = a.out_sw == 1 && a.out_sh % 2 == 0 && a.out_sc % 2 == 0 &&
+              base % (uint64_t)(2 * esz) == 0;
+  a.out_vec4 = a.out_sw == 1 && a.out_sh % 4 == 0 && a.out_sc % 4 == 0 &&
+               base % (uint64_t)(4 * esz) == 0;
+}
+
+// Tile shape of a one-launch forward: `threads` per CTA, `cols` coarse columns
+// per thread (1: 256 or 128 threads, 247 or 119 output columns per strip; 2:
+// 128 or 64 threads, 246 or 118) and coarse rows per band.
+struct FwdPlan {
+  int threads, cols;
+  int64_t rows;
+};
+
+// The plan with the least modelled time for `planes` planes of n x m samples
+// on a GPU of `sms` SMs; threads (with cols) and rows are taken as given where
+// they are not 0.
+FwdPlan fwd_plan_for(int64_t n, int64_t m, int64_t planes, int sms, int threads, int cols,
+                     int64_t rows);
 
 int tile_width_fwd();
 int threads_fwd();

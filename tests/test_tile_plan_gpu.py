@@ -1,0 +1,44 @@
+"""The library's own choice of tile shapes: every plan gives the bits of one
+fixed tile, from a single sample to several waves of CTAs, in the one-launch and
+the batched form."""
+import pytest
+import torch
+
+from paper_2312_00229_gb300 import api
+
+pytestmark = pytest.mark.gpu
+
+
+def _img(shape, seed, dtype=torch.uint8):
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    x = torch.randint(0, 256, shape, generator=g, device="cuda", dtype=torch.uint8)
+    return x if dtype == torch.uint8 else (x.float() * (1.0 / 255.0)).to(dtype)
+
+
+@pytest.mark.parametrize("c,n,m", [(1, 1, 1), (3, 2, 7), (1, 3, 400), (3, 17, 118), (3, 48, 64),
+                                   (1, 119, 119), (2, 200, 247), (3, 333, 500), (1, 1024, 130),
+                                   (65, 40, 246), (3, 700, 900)])
+@pytest.mark.parametrize("mode", [0, 1])
+def test_default_plan_bits(c, n, m, mode):
+    x = _img((c, n, m), 7 * n + m)
+    p = api.Params(out_mode=mode)
+    ref = api.zoom2x_fwd(x, p, rows_per_tile=64, tile_width=247)
+    assert torch.equal(api.zoom2x_fwd(x, p, rows_per_tile=0, tile_width=0), ref)
+    for tw in (118, 119, 246, 247):  # band height chosen for a given width
+        assert torch.equal(api.zoom2x_fwd(x, p, rows_per_tile=0, tile_width=tw), ref)
+    for rows in (1, 2, 5, 33):  # width chosen for a given band height
+        assert torch.equal(api.zoom2x_fwd(x, p, rows_per_tile=rows, tile_width=0), ref)
+
+
+@pytest.mark.parametrize("sides", [[(1, 1)], [(5, 9)] * 3, [(64, 80), (1, 300), (300, 1)],
+                                   [(100 + 7 * i, 90 + 11 * i) for i in range(33)],
+                                   [(16 + i % 5, 20 + i % 3) for i in range(1100)],
+                                   [(900, 700), (8, 8)]])
+def test_batched_default_bits(sides):
+    imgs = [_img((3, n, m), i) for i, (n, m) in enumerate(sides)]
+    for rows, tw in ((0, 0), (0, 119), (0, 246), (24, 0)):
+        outs = api.BatchedPlan(imgs, rows_per_tile=rows, tile_width=tw).run()
+        step = max(1, len(imgs) // 40)
+        for k in range(0, len(imgs), step):
+            ref = api.zoom2x_fwd(imgs[k], rows_per_tile=64, tile_width=247)
+            assert torch.equal(outs[k], ref), (rows, tw, k)
