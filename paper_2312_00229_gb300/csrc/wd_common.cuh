@@ -32,7 +32,8 @@ enum DType { DT_U8 = 0, DT_F16 = 1, DT_BF16 = 2, DT_F32 = 3 };
 //   B2R : beta == 2, alpha = 1 / D^2 as written; chosen by the host only
 //         where the storage type bounds the data so that every weight, their
 //         sum and the blend numerator stay inside the normal FP32 range.
-enum BetaMode { B2 = 0, BGEN = 1, B0 = 2, B2R = 3 };
+//   B1  : beta == 1 (forward kernels of the common storage pairs).
+enum BetaMode { B2 = 0, BGEN = 1, B0 = 2, B2R = 3, B1 = 4 };
 
 // Constants of the method folded for the kernels.  eps_h is spread over the
 // five smoothness indicators that form each D (Eqs. 2DsmoothnessFinal and
@@ -286,6 +287,8 @@ __device__ __forceinline__ float blend4(float D0, float D1, float D2, float D3, 
     // alpha_k = (D_min / D_k)^2: the same weights as 1 / D_k^2 up to a common
     // factor, in range for any data magnitude, and without a branch
     return blend_scale_free(D0, D1, D2, D3, M01, M23, s0, s1, s2, s3, 2.0f);
+  } else if (BMODE == B1) {
+    return blend_scale_free(D0, D1, D2, D3, M01, M23, s0, s1, s2, s3, 1.0f);
   } else if (BMODE == B2R) {
     const float a0 = rcp_approx(D0 * D0), a1 = rcp_approx(D1 * D1);
     const float a2 = rcp_approx(D2 * D2), a3 = rcp_approx(D3 * D3);

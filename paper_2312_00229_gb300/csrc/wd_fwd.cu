@@ -1,7 +1,7 @@
 // Forward 2x zoom, one launch per image (all planes): grid = strips x bands x
 // planes, one CTA per tile.  The tile body is in wd_fwd_tile.cuh.  Storage
-// types are compile-time parameters for the common pairs (wd_fwd_typed.cu);
-// any other pair, and beta != 2, goes through the run-time-typed kernels here.
+// types are compile-time parameters for the common pairs (wd_fwd_typed*.cu);
+// any other pair, and beta = 0, goes through the run-time-typed kernels here.
 #include <cmath>
 
 #include "wd_cascade.h"
@@ -12,6 +12,10 @@ namespace wdweno {
 
 cudaError_t launch_fwd_typed(const FwdArgs& a, const MethodConsts& k, int bmode,
                              cudaStream_t stream, bool* handled);
+cudaError_t launch_fwd_typed_b1(const FwdArgs& a, const MethodConsts& k, cudaStream_t stream,
+                                bool* handled);
+cudaError_t launch_fwd_typed_bgen(const FwdArgs& a, const MethodConsts& k, cudaStream_t stream,
+                                  bool* handled);
 
 int tile_width_fwd() { return fwd_tile::TILE_W; }
 int threads_fwd() { return fwd_tile::THREADS; }
@@ -90,6 +94,12 @@ cudaError_t launch_zoom2x_fwd(const FwdArgs& a, const MethodConsts& k, int bmode
     if (handled) return e;
     if (bmode == B2R) return fwd_kernels::launch_fwd<B2R, DynIO>(a, k, stream);
     return fwd_kernels::launch_fwd<B2, DynIO>(a, k, stream);
+  }
+  if (bmode == BGEN) {
+    bool handled = false;
+    cudaError_t e = k.beta == 1.f ? launch_fwd_typed_b1(a, k, stream, &handled)
+                                  : launch_fwd_typed_bgen(a, k, stream, &handled);
+    if (handled) return e;
   }
   if (bmode == B0) return fwd_kernels::launch_fwd<B0, DynIO>(a, k, stream);
   return fwd_kernels::launch_fwd<BGEN, DynIO>(a, k, stream);

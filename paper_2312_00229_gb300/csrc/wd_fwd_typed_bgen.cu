@@ -1,0 +1,24 @@
+// Forward kernels with the storage types fixed at compile time and
+// any other beta > 0: the same-type pairs.  (The run-time-typed kernels of wd_fwd.cu
+// issue 503 instructions a px-ch, these 250 to 330: 1x1025x1025 FP32 at
+// beta = 1 on the 2n-1 grid, 35.0 -> 18.7 us with the tile plan of wd_fwd_model.h.)
+#include "wd_fwd_kernels.cuh"
+
+namespace wdweno {
+
+cudaError_t launch_fwd_typed_bgen(const FwdArgs& a, const MethodConsts& k, cudaStream_t stream,
+                                  bool* handled) {
+  using fwd_kernels::launch_fwd;
+  using fwd_tile::TypedIO;
+  *handled = a.in_dtype == a.out_dtype;
+  if (!*handled) return cudaSuccess;
+  switch (a.in_dtype) {
+    case DT_U8: return launch_fwd<BGEN, TypedIO<uint8_t, uint8_t>>(a, k, stream);
+    case DT_F16: return launch_fwd<BGEN, TypedIO<__half, __half>>(a, k, stream);
+    case DT_BF16:
+      return launch_fwd<BGEN, TypedIO<__nv_bfloat16, __nv_bfloat16>>(a, k, stream);
+    default: return launch_fwd<BGEN, TypedIO<float, float>>(a, k, stream);
+  }
+}
+
+}  // namespace wdweno

@@ -39,11 +39,12 @@ __device__ __forceinline__ float blend4_pk(float D0, float D1, float D2, float D
     const f2 a23 = pk_rcp(pk_mul(make_float2(D2, D3), make_float2(D2, D3)));
     const float den = (a01.x + a01.y) + (a23.x + a23.y);
     return combine(a01.x, a01.y, a23.x, a23.y, M01, M23, s0, s1, s2, s3, rcp_approx(den + den));
-  } else if (BMODE == B2) {
+  } else if (BMODE == B2 || BMODE == B1) {
     const f2 dmin = pk_bc(fminf(fminf(D0, D1), fminf(D2, D3)));
     const f2 r01 = pk_mul(dmin, pk_rcp(make_float2(D0, D1)));
     const f2 r23 = pk_mul(dmin, pk_rcp(make_float2(D2, D3)));
-    const f2 a01 = pk_mul(r01, r01), a23 = pk_mul(r23, r23);
+    const f2 a01 = BMODE == B1 ? r01 : pk_mul(r01, r01);
+    const f2 a23 = BMODE == B1 ? r23 : pk_mul(r23, r23);
     const float den = (a01.x + a01.y) + (a23.x + a23.y);
     return combine(a01.x, a01.y, a23.x, a23.y, M01, M23, s0, s1, s2, s3, rcp_approx(den + den));
   } else {

@@ -1,6 +1,7 @@
 """The library's own choice of tile shapes: every plan gives the bits of one
 fixed tile, from a single sample to several waves of CTAs, in the one-launch and
-the batched form."""
+the batched form; and the kernels of a fixed storage pair give the bits of the
+run-time-typed ones for beta != 2."""
 import pytest
 import torch
 
@@ -42,3 +43,22 @@ def test_batched_default_bits(sides):
         for k in range(0, len(imgs), step):
             ref = api.zoom2x_fwd(imgs[k], rows_per_tile=64, tile_width=247)
             assert torch.equal(outs[k], ref), (rows, tw, k)
+
+
+@pytest.mark.parametrize("beta", [0.1, 1.0, 1.5, 3.0])
+@pytest.mark.parametrize("n,m,mode", [(37, 130, 0), (64, 246, 1), (5, 3, 0)])
+def test_fixed_types_equal_run_time_types(beta, n, m, mode):
+    p = api.Params(beta=beta, out_mode=mode)
+    u8 = _img((2, n, m), 3)
+    f32 = _img((2, n, m), 3, torch.float32)
+    # uint8 -> FP32 runs the run-time-typed kernel, the same-type pairs do not
+    ref = api.zoom2x_fwd(u8, p, out_dtype=torch.float32, rows_per_tile=16, tile_width=119)
+    for tw in (118, 119, 246, 247):
+        assert torch.equal(api.zoom2x_fwd(f32, p, tile_width=tw, rows_per_tile=0), ref)
+        got = api.zoom2x_fwd(u8, p, tile_width=tw, rows_per_tile=0)
+        assert torch.equal(got, api.zoom2x_fwd(f32, p, out_dtype=torch.uint8, tile_width=119,
+                                               rows_per_tile=16))
+    for dt in (torch.float16, torch.bfloat16):
+        x = _img((2, n, m), 3, dt)
+        ref16 = api.zoom2x_fwd(x.float(), p, rows_per_tile=0).to(dt)
+        assert torch.equal(api.zoom2x_fwd(x, p, rows_per_tile=0), ref16)
