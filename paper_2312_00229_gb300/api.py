@@ -113,6 +113,19 @@ def _out_like(x: torch.Tensor, params: Params, layout: str, dtype) -> torch.Tens
     return torch.empty(shape, dtype=dtype, device=x.device)
 
 
+def _level_out(x: torch.Tensor, params: Params, layout: str, dtype) -> torch.Tensor:
+    """Output image of an inner level of a chain of zooms: as ``_out_like``,
+    with planar rows padded to a multiple of four elements.  Only the next
+    level reads it, and rows that all start on a four-element boundary are
+    written with one vector store per thread and fine row (odd widths of the
+    2n-1 grid otherwise take three)."""
+    if layout == "hwc" or x.dim() < 2:
+        return _out_like(x, params, layout, dtype)
+    h, w = out_hw(x.shape[-2], x.shape[-1], params)
+    return torch.empty((*x.shape[:-2], h, (w + 3) // 4 * 4), dtype=dtype,
+                       device=x.device)[..., :w]
+
+
 def zoom2x_fwd(x: torch.Tensor, params: Optional[Params] = None, out_dtype=None,
                layout: str = "chw", rows_per_tile: Optional[int] = None,
                out: Optional[torch.Tensor] = None, tile_width: int = 0) -> torch.Tensor:
@@ -249,8 +262,11 @@ def cascade_zoom(x: torch.Tensor, levels: int, params: Optional[Params] = None, 
     for lvl in range(levels):
         last = lvl == levels - 1
         p = dataclasses.replace(params, h=params.h / (1 << lvl), data_bound=bounds[lvl])
-        cur = zoom2x_fwd(cur, p, out_dtype=(out_dtype or x.dtype) if last else inter_dtype,
-                         layout=layout)
+        if last:
+            cur = zoom2x_fwd(cur, p, out_dtype=out_dtype or x.dtype, layout=layout)
+        else:
+            cur = zoom2x_fwd(cur, p, layout=layout,
+                             out=_level_out(cur, p, layout, inter_dtype))
     return cur
 
 
@@ -307,7 +323,7 @@ def zoom_to(x: torch.Tensor, out_h: int, out_w: int, params: Optional[Params] = 
     for lvl in range(k):
         cur = zoom2x_fwd(cur, dataclasses.replace(p, h=params.h / (1 << lvl),
                                                   data_bound=bounds[lvl]),
-                         out_dtype=inter_dtype, layout=layout)
+                         layout=layout, out=_level_out(cur, p, layout, inter_dtype))
     return resample(cur, out_h, out_w,
                     dataclasses.replace(params, h=params.h / (1 << k), data_bound=bounds[k]),
                     out_dtype=out_dtype or x.dtype, layout=layout)
@@ -326,7 +342,7 @@ class BatchedPlan:
         self.params = params or Params()
         self.layout = layout
         self.rows_per_tile = int(rows_per_tile)
-        self.tile_width = int(tile_width)  # 0 = 247, or 119 (128-thread CTAs)
+        self.tile_width = int(tile_width)  # 0 = the library's default, 118
         dev = images[0].device
         in_dt = images[0].dtype
         for im in images:

@@ -62,3 +62,21 @@ def test_fixed_types_equal_run_time_types(beta, n, m, mode):
         x = _img((2, n, m), 3, dt)
         ref16 = api.zoom2x_fwd(x.float(), p, rows_per_tile=0).to(dt)
         assert torch.equal(api.zoom2x_fwd(x, p, rows_per_tile=0), ref16)
+
+
+@pytest.mark.parametrize("n,m", [(9, 7), (33, 61), (50, 50)])
+def test_padded_inner_levels(n, m):
+    """Inner levels with padded rows: the chain equals explicit contiguous levels."""
+    x = _img((3, n, m), n)
+    cur, bounds = x, api._level_bounds(x, api.Params(), 3)
+    for lvl in range(3):
+        cur = api.zoom2x_fwd(cur, api.Params(h=0.5 ** lvl, data_bound=bounds[lvl]),
+                             out_dtype=torch.uint8 if lvl == 2 else torch.float32).contiguous()
+    assert torch.equal(api.cascade_zoom(x, 3), cur)
+    y = api.zoom_to(x, 3 * n, 3 * m)
+    cur = x
+    for lvl in range(2):
+        cur = api.zoom2x_fwd(cur, api.Params(h=0.5 ** lvl, data_bound=bounds[lvl], out_mode=1),
+                             out_dtype=torch.float32).contiguous()
+    assert torch.equal(y, api.resample(cur, 3 * n, 3 * m, api.Params(h=0.25, data_bound=bounds[2]),
+                                       out_dtype=torch.uint8))
