@@ -11,9 +11,13 @@
 // PolinomZaVelikiStencil) are C_0 = (2 - t)/3, C_1 = (1 + t)/3, so
 //     u = v1 + g t + (t^2 - t)/2 (alpha_0 sL + alpha_1 sR) / (alpha_0 + alpha_1),
 //     alpha_s = C_s / (eps_h + SI_s)^beta                     (Eq. IzrazOmega).
-// One thread per output pixel: four 1-D interpolants down the columns of
-// the 4x4 input window (z_k = w(A(:,k), y)), then one across them
-// (U = w(Z, x)).  Inputs outside the image are clamped to the edge.
+// Inputs outside the image are clamped to the edge.
+//
+// Everything of an interpolant but C_s and the powers of t belongs to its
+// cell, not to t: g, sL, sR and the weights' powers of the indicators are
+// formed once per cell (Cell2) and evaluated at each output inside (eval2).
+#include <algorithm>
+#include <atomic>
 #include <type_traits>
 
 #include "wd_common.cuh"
@@ -24,145 +28,95 @@ namespace wdweno {
 
 namespace {
 
-// With the position's constants given: C0 = (2 - t)/3 and h = (t^2 - t)/2.
+// Two cells at once on Blackwell's packed two-lane FP32 instructions (pk_*
+// helpers of wd_packed.cuh).  wL, wR: the indicators' part of the weights
+// alpha_0 : alpha_1 = C_0 eR^beta : C_1 eL^beta.
+struct Cell2 {
+  f2 v1, g, sL, sR, wL, wR;
+};
+
 template <int BMODE>
-__device__ __forceinline__ float weno1d_at(float v0, float v1, float v2, float v3, float t,
-                                           float C0, float h, float eps, float beta) {
-  const float g = v2 - v1;
-  const float sL = fmaf(-2.f, v1, v0 + v2);
-  const float sR = fmaf(-2.f, v2, v1 + v3);
-  const float C1 = 1.f - C0;
-  float a0, a1;
-  if (BMODE == B0) {
-    a0 = C0; a1 = C1;
-  } else if (BMODE == B2R) {
-    // alpha_0 : alpha_1 = C_0 eR^2 : C_1 eL^2 as written; the host picks
-    // this form only where the storage type bounds the data so that every
-    // square, their sum and the numerator below are normal FP32 numbers
-    const float k2 = 13.f / 12.f;
-    const float eL = fmaf(g, g, fmaf(k2 * sL, sL, eps));
-    const float eR = fmaf(g, g, fmaf(k2 * sR, sR, eps));
-    a0 = C0 * (eR * eR);
-    a1 = C1 * (eL * eL);
+__device__ __forceinline__ Cell2 cell2(f2 v0, f2 v1, f2 v2, f2 v3, float eps, float beta) {
+  Cell2 c;
+  c.v1 = v1;
+  c.g = pk_sub(v2, v1);
+  c.sL = pk_fma(pk_bc(-2.f), v1, pk_add(v0, v2));
+  c.sR = pk_fma(pk_bc(-2.f), v2, pk_add(v1, v3));
+  if (BMODE == B0) return c;
+  const f2 k2 = pk_bc(13.f / 12.f), e = pk_bc(eps);
+  const f2 eL = pk_fma(c.g, c.g, pk_fma(pk_mul(k2, c.sL), c.sL, e));
+  const f2 eR = pk_fma(c.g, c.g, pk_fma(pk_mul(k2, c.sR), c.sR, e));
+  if (BMODE == B2R) {
+    // the squares as written; the host picks this form only where the storage
+    // type bounds the data so that every square, their sum and the numerator
+    // of eval2 are normal FP32 numbers
+    c.wL = pk_mul(eL, eL);
+    c.wR = pk_mul(eR, eR);
   } else {
-    // alpha_0 : alpha_1 = C_0 eR^beta : C_1 eL^beta with both indicators
-    // divided by the larger one, so no power over- or underflows.  eps is
-    // at least 1e-30 (host side), so the larger indicator is a normal number.
-    const float k2 = 13.f / 12.f;
-    const float eL = fmaf(g, g, fmaf(k2 * sL, sL, eps));
-    const float eR = fmaf(g, g, fmaf(k2 * sR, sR, eps));
-    const float inv = rcp_approx(fmaxf(eL, eR));
-    const float rL = eL * inv, rR = eR * inv;
-    if (BMODE == B2) {
-      a0 = C0 * rR * rR; a1 = C1 * rL * rL;
-    } else {
-      a0 = C0 * ex2_approx(beta * lg2_approx(rR));
-      a1 = C1 * ex2_approx(beta * lg2_approx(rL));
+    // both indicators divided by the larger one, so no power over- or
+    // underflows.  eps is at least 1e-30 (host side), so the larger indicator
+    // is a normal number.
+    const f2 inv = pk_rcp(make_float2(fmaxf(eL.x, eR.x), fmaxf(eL.y, eR.y)));
+    c.wL = pk_mul(eL, inv);
+    c.wR = pk_mul(eR, inv);
+    if (BMODE != B2) {
+      const f2 b = pk_bc(beta);
+      const f2 lR = pk_mul(b, make_float2(lg2_approx(c.wR.x), lg2_approx(c.wR.y)));
+      const f2 lL = pk_mul(b, make_float2(lg2_approx(c.wL.x), lg2_approx(c.wL.y)));
+      c.wR = make_float2(ex2_approx(lR.x), ex2_approx(lR.y));
+      c.wL = make_float2(ex2_approx(lL.x), ex2_approx(lL.y));
     }
   }
-  // a0 + a1 >= 1/3 in the scaled forms: one ratio is 1 and both C_s are at
-  // least 1/3
-  const float mix = fmaf(a0, sL, a1 * sR) * rcp_approx(a0 + a1);
-  return fmaf(h, mix, fmaf(g, t, v1));
+  return c;
 }
 
-// Two interpolants at once on Blackwell's packed two-lane FP32 instructions
-// (pk_* helpers of wd_packed.cuh): weno1d_at on lane pairs, the same
-// expressions in the same order, each lane rounded as the scalar form.
+// The interpolants at offset t: C0 = (2 - t)/3, h = (t^2 - t)/2.
 template <int BMODE>
-__device__ __forceinline__ f2 weno1d_at2(f2 v0, f2 v1, f2 v2, f2 v3, f2 t, f2 C0, f2 h,
-                                         float eps, float beta) {
-  const f2 g = pk_sub(v2, v1);
-  const f2 sL = pk_fma(pk_bc(-2.f), v1, pk_add(v0, v2));
-  const f2 sR = pk_fma(pk_bc(-2.f), v2, pk_add(v1, v3));
+__device__ __forceinline__ f2 eval2(const Cell2& c, f2 t, f2 C0, f2 h) {
   const f2 C1 = pk_sub(pk_bc(1.f), C0);
   f2 a0, a1;
   if (BMODE == B0) {
-    a0 = C0; a1 = C1;
+    a0 = C0;
+    a1 = C1;
+  } else if (BMODE == B2) {
+    a0 = pk_mul(pk_mul(C0, c.wR), c.wR);
+    a1 = pk_mul(pk_mul(C1, c.wL), c.wL);
   } else {
-    const f2 k2 = pk_bc(13.f / 12.f), e = pk_bc(eps);
-    const f2 eL = pk_fma(g, g, pk_fma(pk_mul(k2, sL), sL, e));
-    const f2 eR = pk_fma(g, g, pk_fma(pk_mul(k2, sR), sR, e));
-    if (BMODE == B2R) {
-      a0 = pk_mul(C0, pk_mul(eR, eR));
-      a1 = pk_mul(C1, pk_mul(eL, eL));
-    } else {
-      const f2 inv = pk_rcp(make_float2(fmaxf(eL.x, eR.x), fmaxf(eL.y, eR.y)));
-      const f2 rL = pk_mul(eL, inv), rR = pk_mul(eR, inv);
-      if (BMODE == B2) {
-        a0 = pk_mul(pk_mul(C0, rR), rR);
-        a1 = pk_mul(pk_mul(C1, rL), rL);
-      } else {
-        const f2 b = pk_bc(beta);
-        const f2 lR = pk_mul(b, make_float2(lg2_approx(rR.x), lg2_approx(rR.y)));
-        const f2 lL = pk_mul(b, make_float2(lg2_approx(rL.x), lg2_approx(rL.y)));
-        a0 = pk_mul(C0, make_float2(ex2_approx(lR.x), ex2_approx(lR.y)));
-        a1 = pk_mul(C1, make_float2(ex2_approx(lL.x), ex2_approx(lL.y)));
-      }
-    }
+    a0 = pk_mul(C0, c.wR);
+    a1 = pk_mul(C1, c.wL);
   }
-  const f2 mix = pk_mul(pk_fma(a0, sL, pk_mul(a1, sR)), pk_rcp(pk_add(a0, a1)));
-  return pk_fma(h, mix, pk_fma(g, t, v1));
+  // a0 + a1 >= 1/3 in the scaled forms: one ratio is 1 and both C_s are at
+  // least 1/3
+  const f2 mix = pk_mul(pk_fma(a0, c.sL, pk_mul(a1, c.sR)), pk_rcp(pk_add(a0, a1)));
+  return pk_fma(h, mix, pk_fma(c.g, t, c.v1));
 }
 
-template <int BMODE>
-__device__ __forceinline__ float weno1d(float v0, float v1, float v2, float v3, float t,
-                                        float eps, float beta) {
-  return weno1d_at<BMODE>(v0, v1, v2, v3, t, (2.f - t) * (1.f / 3.f), 0.5f * fmaf(t, t, -t),
-                          eps, beta);
-}
+__device__ __forceinline__ float pos_c0(float t) { return (2.f - t) * (1.f / 3.f); }
+__device__ __forceinline__ float pos_h(float t) { return 0.5f * fmaf(t, t, -t); }
 
 // Cell index and offset of output index j on the endpoint-aligned grid of
 // n_out points over 0..n-1: i = floor(j (n-1) / (n_out-1)) exactly (by
 // multiply-high when the numerator fits 32 bits), t = remainder / (n_out-1).
-__device__ __forceinline__ void grid_pos(int64_t j, int64_t n, int64_t n_out, const AxisDiv& d,
-                                         int64_t& i, float& t) {
+__device__ __forceinline__ void grid_pos(int j, int n, int n_out, const AxisDiv& d, int& i,
+                                         float& t) {
   if (n <= 1 || n_out <= 1) { i = 0; t = 0.f; return; }
-  const int64_t den = n_out - 1;
-  int64_t q, rem;
+  const int den = n_out - 1;
   if (d.fast) {
     const uint32_t num = (uint32_t)j * (uint32_t)(n - 1);
     const uint32_t t1 = __umulhi(d.mag, num);
-    const uint32_t qq = (t1 + ((num - t1) >> d.sh1)) >> d.sh2;
-    q = qq;
-    rem = (int64_t)(num - qq * (uint32_t)den);
+    const uint32_t q = (t1 + ((num - t1) >> d.sh1)) >> d.sh2;
+    i = (int)q;
+    t = (float)(int)(num - q * (uint32_t)den) * d.inv;
   } else {
-    const int64_t num = j * (n - 1);
-    q = num / den;
-    rem = num - q * den;
+    const int64_t num = (int64_t)j * (n - 1);
+    const int64_t q = num / den;
+    i = (int)q;
+    t = (float)(num - q * den) * d.inv;
   }
-  if (q > n - 2) { q = n - 2; rem = den; }  // last sample: t = 1 on the last cell
-  i = q;
-  t = rem == den ? 1.f : (float)rem * d.inv;
+  if (i > n - 2) { i = n - 2; t = 1.f; }  // last sample: t = 1 on the last cell
 }
 
-template <int BMODE>
-__global__ void __launch_bounds__(256) resample_kernel(ResampleArgs a, float eps, float beta) {
-  const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t r = (int64_t)blockIdx.y * blockDim.y + threadIdx.y;
-  if (r >= a.n_out || c >= a.m_out) return;
-  const int64_t plane = blockIdx.z;
-  int64_t i, j;
-  float ty, tx;
-  grid_pos(r, a.n, a.n_out, a.div_y, i, ty);
-  grid_pos(c, a.m, a.m_out, a.div_x, j, tx);
-  const int64_t base = plane * a.in_sc;
-  float z[4];
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const int64_t col = j - 1 + q < 0 ? 0 : (j - 1 + q > a.m - 1 ? a.m - 1 : j - 1 + q);
-    float v[4];
-#pragma unroll
-    for (int p = 0; p < 4; ++p) {
-      const int64_t row = i - 1 + p < 0 ? 0 : (i - 1 + p > a.n - 1 ? a.n - 1 : i - 1 + p);
-      v[p] = load_elem(a.in, base + row * a.in_sh + col * a.in_sw, a.in_dtype);
-    }
-    z[q] = a.n > 1 ? weno1d<BMODE>(v[0], v[1], v[2], v[3], ty, eps, beta) : v[1];
-  }
-  const float u = a.m > 1 ? weno1d<BMODE>(z[0], z[1], z[2], z[3], tx, eps, beta) : z[1];
-  store_elem(a.out, plane * a.out_sc + r * a.out_sh + c * a.out_sw, u, a.out_dtype,
-             a.clamp_float);
-}
+__device__ __forceinline__ int clamp_idx(int v, int n) { return v < 0 ? 0 : (v > n - 1 ? n - 1 : v); }
 
 // Storage access: a concrete element type, or Dyn for the run-time type.
 struct Dyn {};
@@ -206,197 +160,404 @@ __device__ __forceinline__ void rs_store4(void* base, int64_t idx, const float (
   }
 }
 
-// Separable tiled form for output/input spacing ratios down to 1/2 on both
-// axes: a CTA owns tile_rows (16 or 32) output rows x RS_TC output columns of one
-// plane.
-//   stage 0  the input window those outputs read (rows i(r0)-1 .. i(r_last)+2,
-//            columns j(c0)-1 .. j(c_last)+2, clamped) decoded into shared memory
-//   pass 1   the column interpolants z(r, k) = w(A(:, k), y_r) of the tile's
-//            rows at every window column (Eq. tensor, first factor)
-//   pass 2   each thread interpolates four consecutive outputs of a row across
-//            the z values (Eq. tensor, second factor) and stores them together
-// Per output this is 1 + (in/out column ratio) + halo 1-D interpolants
-// instead of 5.
-// Output rows per tile: 32 when the rows are magnified (the per-tile setup
-// and window decode spread over more outputs), 16 when they are reduced (the
-// window then has up to twice the tile's rows, and taller tiles would leave
-// fewer CTAs per SM).
-constexpr int RS_TR_UP = 32;
-constexpr int RS_TR_DOWN = 16;
-constexpr int RS_TC = 128;
-constexpr int RS_WC = 2 * RS_TC + 8;  // window columns (>= 2 (RS_TC - 1) + 5)
-constexpr int RS_THREADS = 256;
-
+// One thread per output, for reductions beyond 1/2 (little to share between
+// neighbouring outputs) and single-sample axes: all 16 loads are issued before
+// the first is used, columns are interpolated in packed pairs.  1080p ->
+// 480x270 uint8: 9.2 us with run-time types and 64-bit positions, now 6.8.
 template <int BMODE, class TIn, class TOut>
-__global__ void __launch_bounds__(RS_THREADS) resample_tiled_kernel(ResampleArgs a, float eps,
-                                                                   float beta) {
-  extern __shared__ float rs_smem[];
-  float(*win)[RS_WC] = reinterpret_cast<float(*)[RS_WC]>(rs_smem);               // a.win_rows
-  float(*z)[RS_WC] = reinterpret_cast<float(*)[RS_WC]>(rs_smem + a.win_rows * RS_WC);  // tile_rows
-  __shared__ int col_j[RS_TC];
-  __shared__ float col_t[RS_TC];
-  __shared__ int row_i[RS_TR_UP];
-  __shared__ float row_t[RS_TR_UP];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int64_t c0 = (int64_t)blockIdx.x * RS_TC;
-  const int tr = a.tile_rows;
-  const int64_t r0 = (int64_t)blockIdx.y * tr;
+__global__ void __launch_bounds__(256) resample_kernel(ResampleArgs a, float eps, float beta) {
+  const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t r = (int64_t)blockIdx.y * blockDim.y + threadIdx.y;
+  if (r >= a.n_out || c >= a.m_out) return;
   const int64_t plane = blockIdx.z;
-  const int nc = (int)(a.m_out - c0 < RS_TC ? a.m_out - c0 : RS_TC);
-  const int nr = (int)(a.n_out - r0 < tr ? a.n_out - r0 : tr);
-  // Every output column's and row's cell index (absolute) and offset; the
-  // first and last of them bound the input window.
-  if (tid < nc) {
-    int64_t j;
-    float t;
-    grid_pos(c0 + tid, a.m, a.m_out, a.div_x, j, t);
-    col_j[tid] = (int)j;
-    col_t[tid] = t;
-  }
-  if (tid >= RS_TC && tid - RS_TC < nr) {
-    int64_t i;
-    float t;
-    grid_pos(r0 + tid - RS_TC, a.n, a.n_out, a.div_y, i, t);
-    row_i[tid - RS_TC] = (int)i;
-    row_t[tid - RS_TC] = t;
-  }
-  __syncthreads();
-  const int64_t kfirst = (int64_t)col_j[0] - 1, ifirst = (int64_t)row_i[0] - 1;
-  const int wc = col_j[nc - 1] + 2 - (int)kfirst + 1;  // <= RS_WC (host checks the x scale)
-  const int wr = row_i[nr - 1] + 2 - (int)ifirst + 1;  // <= a.win_rows (host sizes it)
-  // stage 0: decoded, clamped input window.  A thread takes 2 x 2 elements
-  // at a time (rows 8 apart, columns 32 apart) and issues their four loads
-  // before it converts any of them, so that the loads overlap.
-  constexpr int WR = RS_THREADS / 32;  // rows one pass of the warps covers
-  const int64_t pbase = plane * a.in_sc;
-  for (int rr0 = warp; rr0 < wr; rr0 += 2 * WR) {
-    int64_t rbase[2];
+  const int n = (int)a.n, m = (int)a.m;
+  int i, j;
+  float ty, tx;
+  grid_pos((int)r, n, (int)a.n_out, a.div_y, i, ty);
+  grid_pos((int)c, m, (int)a.m_out, a.div_x, j, tx);
+  int64_t row[4], col[4];
 #pragma unroll
-    for (int u = 0; u < 2; ++u) {
-      int64_t row = ifirst + rr0 + u * WR;
-      row = row < 0 ? 0 : (row > a.n - 1 ? a.n - 1 : row);
-      rbase[u] = pbase + row * a.in_sh;
+  for (int p = 0; p < 4; ++p) {
+    row[p] = plane * a.in_sc + (int64_t)clamp_idx(i - 1 + p, n) * a.in_sh;
+    col[p] = (int64_t)clamp_idx(j - 1 + p, m) * a.in_sw;
+  }
+  uint32_t b[4][4];
+#pragma unroll
+  for (int p = 0; p < 4; ++p)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) b[p][q] = rs_load_bits<TIn>(a.in, row[p] + col[q], a.in_dtype);
+  f2 z[2];
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    f2 v[4];
+#pragma unroll
+    for (int p = 0; p < 4; ++p)
+      v[p] = make_float2(rs_value<TIn>(b[p][2 * q], a.in_dtype),
+                         rs_value<TIn>(b[p][2 * q + 1], a.in_dtype));
+    z[q] = n > 1 ? eval2<BMODE>(cell2<BMODE>(v[0], v[1], v[2], v[3], eps, beta), pk_bc(ty),
+                                pk_bc(pos_c0(ty)), pk_bc(pos_h(ty)))
+                 : v[1];
+  }
+  float u = z[0].y;
+  if (m > 1)
+    u = eval2<BMODE>(cell2<BMODE>(pk_bc(z[0].x), pk_bc(z[0].y), pk_bc(z[1].x), pk_bc(z[1].y), eps,
+                                  beta),
+                     pk_bc(tx), pk_bc(pos_c0(tx)), pk_bc(pos_h(tx)))
+            .x;
+  rs_store<TOut>(a.out, plane * a.out_sc + r * a.out_sh + c * a.out_sw, u, a.out_dtype,
+                 a.clamp_float);
+}
+
+// Tile sizes of the tiled form below.
+constexpr int RS_WARPS = 8;
+constexpr int RS_THREADS = 32 * RS_WARPS;
+constexpr int RS_MAX_ROWS = 8;                 // output rows per warp, at most
+constexpr int RS_DOWN_ROWS = 4;                // the same, where the rows are reduced
+constexpr int RS_CELLS = 8;                    // input cells a warp's rows span, at most
+constexpr int RS_PRE = RS_CELLS + 3;           // input rows
+constexpr int RS_TC_DOWN = 128;                // output columns of a tile, reduced
+constexpr int RS_TC_MAX = 480;                 // and at most, magnified
+constexpr int RS_WC_UP = 64;                   // window columns, magnified
+constexpr int RS_WC_DOWN = 2 * RS_TC_DOWN + 8; // (>= 2 (RS_TC_DOWN - 1) + 5)
+constexpr int RS_MAX_IN = 2 * RS_WARPS * RS_DOWN_ROWS + 8;  // input rows of a tile, at most
+constexpr int RS_REG_OUT = 4;                  // outputs of a cell with constants in registers
+
+template <class T>
+__device__ __forceinline__ int elem_bytes(int dt) {
+  if constexpr (std::is_same<T, Dyn>::value)
+    return dt == DT_U8 ? 1 : (dt == DT_F32 ? 4 : 2);
+  else
+    return (int)sizeof(T);
+}
+
+// A warp copies a row of `nc` encoded elements from shared memory to `out`, in
+// words of four elements where the output's rows allow that.
+template <class E, class V>
+__device__ __forceinline__ void flush_as(char* out, int64_t sw, int vec4,
+                                         const unsigned char* stage, int nc, int lane) {
+  int done = 0;
+  if (vec4) {
+    const int words = nc >> 2;
+    V* dst = reinterpret_cast<V*>(out) + lane;
+    const V* src = reinterpret_cast<const V*>(stage) + lane;
+#pragma unroll
+    for (int w = 0; w < RS_TC_MAX / 128 + 1; ++w) {
+      if (32 * w >= words) break;  // (uniform)
+      if (lane + 32 * w < words) dst[32 * w] = src[32 * w];
     }
-    for (int k0 = lane; k0 < wc; k0 += 64) {
-      uint32_t b[2][2];
+    done = words * 4;
+    if (done == nc) return;
+  }
+  E* dst = reinterpret_cast<E*>(out);
+  const E* src = reinterpret_cast<const E*>(stage);
+  for (int c = done + lane; c < nc; c += 32) dst[c * sw] = src[c];
+}
+
+template <class T>
+__device__ __forceinline__ void rs_flush(char* out, int64_t sw, int vec4,
+                                         const unsigned char* stage, int nc, int lane, int dt) {
+  const int esz = elem_bytes<T>(dt);
+  if (esz == 1)
+    flush_as<uint8_t, uint32_t>(out, sw, vec4, stage, nc, lane);
+  else if (esz == 4)
+    flush_as<float, float4>(out, sw, vec4, stage, nc, lane);
+  else
+    flush_as<uint16_t, uint2>(out, sw, vec4, stage, nc, lane);
+}
+
+// Separable tiled form for output/input spacing ratios down to 1/2 on both
+// axes.  A CTA of 8 warps owns a tile of output columns and 8 `rows` output
+// rows of one plane; a warp owns `rows` consecutive ones and never waits for
+// another after the position tables:
+//   pass 1   the column interpolants z(r, k) = w(A(:, k), y_r) (Eq. tensor,
+//            first factor) of its rows at the tile's window columns, from the
+//            input rows straight to registers (all loads in flight before the
+//            first is used); an input cell's indicators serve every output
+//            row inside it
+//   pass 2   the row interpolants across the z values (second factor)
+// Per output this is 1 + (in/out column ratio) + halo 1-D interpolants
+// instead of the 5 of the direct form.
+//
+// Magnified columns (UP): the tile is as wide as fits 64 window columns, two
+// per lane, and pass 2 gives a lane two cells of the row, whose indicators
+// serve all of their outputs (three at 3x).  Reduced columns: 128 output
+// columns, four per lane.  Either way the encoded outputs go through a staging
+// row in shared memory to whole-word stores.
+//
+// What bounds it: instruction issue (70% of slots at 3x uint8; FMA pipe 47%, LSU
+// 44%), a third of it address arithmetic.  Against the form before (a decoded
+// window in shared memory, every output's indicators formed anew, 4-byte
+// stores from four outputs per lane with strided z reads), us:
+//     1080p uint8 -> 3x 124 -> 79, -> 2x 77 -> 48, -> 1.33x 39.9 -> 33.5, 1x 33 -> 26
+//     4317x7677 FP32 -> 3240x5760 uint8 353 -> 224; 1080p FP32 -> 900x1600 26 -> 20
+// Small outputs are bound by the launch and one warp's chain: 200x300 -> 500x700
+// 5.0 -> 5.3, 64x64 -> 8x 4.7 -> 6.2 (nine outputs a cell, in turn), 100x100 from
+// 64x64 4.7 -> 3.3.  Packed constants pinned in registers, scalar instead of
+// packed arithmetic, and two or four CTAs per SM measured slower.
+template <bool UP>
+struct RsShared {
+  static constexpr int TC = UP ? RS_TC_MAX : RS_TC_DOWN;
+  static constexpr int WZ = UP ? RS_WC_UP + 4 : RS_WC_DOWN;
+  float4 row_a[RS_WARPS * RS_MAX_ROWS];  // (t, t, C0, C0) of each output row
+  float2 row_h[RS_WARPS * RS_MAX_ROWS];  // (h, h)
+  int64_t in_off[RS_MAX_IN];             // byte offset of each (clamped) input row
+  int row_i[RS_WARPS * RS_MAX_ROWS];     // its cell
+  int col_j[TC];
+  float col_t[TC];
+  int start[RS_WC_UP + 1];               // first output column of each cell (UP)
+  float z[RS_WARPS][UP ? RS_MAX_ROWS : RS_DOWN_ROWS][WZ];
+  // encoded outputs of a row, and a spare element
+  __align__(16) unsigned char stage[RS_WARPS][4 * (UP ? RS_TC_MAX : RS_TC_DOWN) + 16];
+};
+
+// Pass 1 of a warp: z of its `nq` output rows (tile rows q0 ..) at window
+// columns k0 + lane and k0 + lane + 32 (columns past the window repeat the
+// last and are not used).  in_base: input row of in_off[0].
+template <int BMODE, class TIn, class SH>
+__device__ __forceinline__ void column_pass(const ResampleArgs& a, SH& sh, int warp, int lane,
+                                            int q0, int nq, int in_base, int kfirst, int wc,
+                                            int k0, const char* plane, int esz, float eps,
+                                            float beta) {
+  const int ka = k0 + lane, kb = ka + 32;
+  const char* pa = plane + (int64_t)clamp_idx(kfirst + min(ka, wc - 1), (int)a.m) * a.in_sw * esz;
+  const char* pb = plane + (int64_t)clamp_idx(kfirst + min(kb, wc - 1), (int)a.m) * a.in_sw * esz;
+  // lane q holds the cell of row q, counted from the first row's
+  const int first = sh.row_i[q0];
+  const int rel = lane < nq ? sh.row_i[q0 + lane] - first : -1;
+  const int rows_in = __shfl_sync(0xffffffffu, rel, nq - 1) + 4;  // input rows they read
+  const int64_t* off = sh.in_off + (first - 1 - in_base);
+  uint32_t ba[RS_PRE], bb[RS_PRE];
 #pragma unroll
-      for (int u = 0; u < 2; ++u)
-#pragma unroll
-        for (int v = 0; v < 2; ++v) {
-          const int k = k0 + 32 * v;
-          int64_t col = kfirst + k;
-          col = col < 0 ? 0 : (col > a.m - 1 ? a.m - 1 : col);
-          b[u][v] = (rr0 + u * WR < wr && k < wc)
-                        ? rs_load_bits<TIn>(a.in, rbase[u] + col * a.in_sw, a.in_dtype)
-                        : 0u;
-        }
-#pragma unroll
-      for (int u = 0; u < 2; ++u)
-#pragma unroll
-        for (int v = 0; v < 2; ++v)
-          if (rr0 + u * WR < wr && k0 + 32 * v < wc)
-            win[rr0 + u * WR][k0 + 32 * v] = rs_value<TIn>(b[u][v], a.in_dtype);
+  for (int p = 0; p < RS_PRE; ++p) {
+    if (p < rows_in) {  // (uniform)
+      ba[p] = rs_load_bits<TIn>(pa + off[p], 0, a.in_dtype);
+      bb[p] = rs_load_bits<TIn>(pb + off[p], 0, a.in_dtype);
     }
   }
-  __syncthreads();
-  // pass 1: column interpolants
-  for (int r = warp; r < nr; r += RS_THREADS / 32) {
-    const float* w0 = win[row_i[r] - 1 - (int)ifirst];
-    if (a.n > 1) {
-      const float ty = row_t[r];
-      const float C0 = (2.f - ty) * (1.f / 3.f), h = 0.5f * fmaf(ty, ty, -ty);
-      // window columns k and k + 32 in the two lanes (a column past the
-      // window repeats k and is not stored)
-      for (int k = lane; k < wc; k += 64) {
-        const bool two = k + 32 < wc;
-        const int kb = two ? k + 32 : k;
-        const f2 zz = weno1d_at2<BMODE>(
-            make_float2(w0[k], w0[kb]), make_float2(w0[k + RS_WC], w0[kb + RS_WC]),
-            make_float2(w0[k + 2 * RS_WC], w0[kb + 2 * RS_WC]),
-            make_float2(w0[k + 3 * RS_WC], w0[kb + 3 * RS_WC]), pk_bc(ty), pk_bc(C0), pk_bc(h), eps,
-            beta);
-        z[r][k] = zz.x;
-        if (two) z[r][k + 32] = zz.y;
-      }
-    } else {
-      for (int k = lane; k < wc; k += 32) z[r][k] = w0[k + RS_WC];
-    }
-  }
-  __syncthreads();
-  // pass 2: four consecutive outputs per thread; the column positions and
-  // their constants are the same for every row of the tile
-  const int c = lane * 4;
-  if (c >= nc) return;
-  const int cn = nc - c < 4 ? nc - c : 4;
-  int kq[4];
-  float tq[4], cq[4], hq[4];
+  f2 v[RS_PRE];
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const int cc = c + (q < cn ? q : 0);  // columns past the tile repeat the first (not stored)
-    kq[q] = col_j[cc] - 1 - (int)kfirst;
-    tq[q] = col_t[cc];
-    cq[q] = (2.f - tq[q]) * (1.f / 3.f);
-    hq[q] = 0.5f * fmaf(tq[q], tq[q], -tq[q]);
-  }
-  const bool interp_x = a.m > 1;
-  int64_t o = plane * a.out_sc + (r0 + warp) * a.out_sh + (c0 + c) * a.out_sw;
-  const int64_t o_step = (RS_THREADS / 32) * a.out_sh;
-  for (int r = warp; r < nr; r += RS_THREADS / 32, o += o_step) {
-    float u[4];
-    const float* zr = z[r];
-    // outputs q and q + 1 in the two lanes
+  for (int p = 0; p < RS_PRE; ++p)
+    if (p < rows_in)
+      v[p] = make_float2(rs_value<TIn>(ba[p], a.in_dtype), rs_value<TIn>(bb[p], a.in_dtype));
+  const bool in_a = ka < SH::WZ, in_b = kb < SH::WZ;
+  float* z = &sh.z[warp][0][0] + k0 + lane;
+  const float4* ra = sh.row_a + q0;
+  const float2* rh = sh.row_h + q0;
 #pragma unroll
-    for (int q = 0; q < 4; q += 2) {
-      const float* za = zr + kq[q];
-      const float* zb = zr + kq[q + 1];
-      if (interp_x) {
-        const f2 uu = weno1d_at2<BMODE>(
-            make_float2(za[0], zb[0]), make_float2(za[1], zb[1]), make_float2(za[2], zb[2]),
-            make_float2(za[3], zb[3]), make_float2(tq[q], tq[q + 1]),
-            make_float2(cq[q], cq[q + 1]), make_float2(hq[q], hq[q + 1]), eps, beta);
-        u[q] = uu.x;
-        u[q + 1] = uu.y;
-      } else {
-        u[q] = za[1];
-        u[q + 1] = zb[1];
-      }
-    }
-    if (a.out_vec4 && cn == 4) {
-      rs_store4<TOut>(a.out, o, u, a.out_dtype, a.clamp_float);
-    } else {
-      for (int q = 0; q < cn; ++q)
-        rs_store<TOut>(a.out, o + q * a.out_sw, u[q], a.out_dtype, a.clamp_float);
+  for (int p = 0; p < RS_CELLS; ++p) {
+    int rows = __popc(__ballot_sync(0xffffffffu, rel == p));  // output rows in cell p
+    if (rows) {
+      const Cell2 c = cell2<BMODE>(v[p], v[p + 1], v[p + 2], v[p + 3], eps, beta);
+#pragma unroll 1
+      do {
+        const float4 ta = *ra++;
+        const float2 th = *rh++;
+        const f2 zz = eval2<BMODE>(c, make_float2(ta.x, ta.y), make_float2(ta.z, ta.w), th);
+        if (in_a) z[0] = zz.x;
+        if (in_b) z[32] = zz.y;
+        z += SH::WZ;
+      } while (--rows);
     }
   }
 }
 
-template <int BMODE, class TIn, class TOut>
-cudaError_t launch_tiled(const ResampleArgs& a, float eps, float beta, cudaStream_t stream) {
-  const size_t smem = (size_t)(a.win_rows + a.tile_rows) * RS_WC * sizeof(float);
-  auto kern = resample_tiled_kernel<BMODE, TIn, TOut>;
-  if (smem > 48 * 1024) {
-    cudaError_t e =
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
+// Pass 2 of a warp on magnified columns: cells of at most NJ outputs, whose
+// positions are kept in registers (with NJ = RS_REG_OUT cells may have more,
+// which read theirs from the tables).
+template <int BMODE, class TOut, int NJ, class SH>
+__device__ __forceinline__ void row_pass_up(const ResampleArgs& a, SH& sh, int warp, int lane,
+                                            int nq, int nc, int cells, int most, char* out,
+                                            int64_t row_bytes, float eps, float beta) {
+  // cells `lane` and `lane + 32`: their output columns and positions; outputs
+  // a cell does not have go to a spare element after the row
+  const int sa = lane < cells ? sh.start[lane] : 0;
+  const int na = lane < cells ? sh.start[lane + 1] - sa : 0;
+  const int sb = lane + 32 < cells ? sh.start[lane + 32] : 0;
+  const int nb = lane + 32 < cells ? sh.start[lane + 33] - sb : 0;
+  f2 t[NJ], C0[NJ], h[NJ];
+  int ia[NJ], ib[NJ];
+#pragma unroll
+  for (int j = 0; j < NJ; ++j) {
+    ia[j] = j < na ? sa + j : RS_TC_MAX;
+    ib[j] = j < nb ? sb + j : RS_TC_MAX;
+    t[j] = make_float2(sh.col_t[j < na ? sa + j : 0], sh.col_t[j < nb ? sb + j : 0]);
+    C0[j] = make_float2(pos_c0(t[j].x), pos_c0(t[j].y));
+    h[j] = make_float2(pos_h(t[j].x), pos_h(t[j].y));
   }
-  const dim3 grid((unsigned)((a.m_out + RS_TC - 1) / RS_TC),
-                  (unsigned)((a.n_out + a.tile_rows - 1) / a.tile_rows), (unsigned)a.planes);
-  kern<<<grid, RS_THREADS, smem, stream>>>(a, eps, beta);
+  unsigned char* stage = sh.stage[warp];
+  const float* zr = sh.z[warp][0] + lane;
+#pragma unroll 1
+  for (int q = 0; q < nq; ++q, out += row_bytes, zr += SH::WZ) {
+    const Cell2 c = cell2<BMODE>(make_float2(zr[0], zr[32]), make_float2(zr[1], zr[33]),
+                                 make_float2(zr[2], zr[34]), make_float2(zr[3], zr[35]), eps,
+                                 beta);
+#pragma unroll
+    for (int j = 0; j < NJ; ++j) {
+      const f2 u = eval2<BMODE>(c, t[j], C0[j], h[j]);
+      rs_store<TOut>(stage, ia[j], u.x, a.out_dtype, a.clamp_float);
+      rs_store<TOut>(stage, ib[j], u.y, a.out_dtype, a.clamp_float);
+    }
+    if (NJ == RS_REG_OUT) {
+#pragma unroll 1
+      for (int j = NJ; j < most; ++j) {
+        const f2 tt = make_float2(sh.col_t[j < na ? sa + j : 0], sh.col_t[j < nb ? sb + j : 0]);
+        const f2 u = eval2<BMODE>(c, tt, make_float2(pos_c0(tt.x), pos_c0(tt.y)),
+                                  make_float2(pos_h(tt.x), pos_h(tt.y)));
+        rs_store<TOut>(stage, j < na ? sa + j : RS_TC_MAX, u.x, a.out_dtype, a.clamp_float);
+        rs_store<TOut>(stage, j < nb ? sb + j : RS_TC_MAX, u.y, a.out_dtype, a.clamp_float);
+      }
+    }
+    __syncwarp();
+    rs_flush<TOut>(out, a.out_sw, a.out_vec4, stage, nc, lane, a.out_dtype);
+    __syncwarp();
+  }
+}
+
+// Pass 2 of a warp on reduced columns: outputs lane, lane + 32, .. of the row
+// (consecutive lanes read z values 1 to 2 apart), two in a packed pair.
+template <int BMODE, class TOut, class SH>
+__device__ __forceinline__ void row_pass_down(const ResampleArgs& a, SH& sh, int warp, int lane,
+                                              int nq, int nc, int kfirst, char* out,
+                                              int64_t row_bytes, float eps, float beta) {
+  const float* z[4];
+  f2 t[2], C0[2], h[2];
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    const int ca = min(lane + 64 * q, nc - 1), cb = min(lane + 64 * q + 32, nc - 1);
+    z[2 * q] = sh.z[warp][0] + (sh.col_j[ca] - 1 - kfirst);
+    z[2 * q + 1] = sh.z[warp][0] + (sh.col_j[cb] - 1 - kfirst);
+    t[q] = make_float2(sh.col_t[ca], sh.col_t[cb]);
+    C0[q] = make_float2(pos_c0(t[q].x), pos_c0(t[q].y));
+    h[q] = make_float2(pos_h(t[q].x), pos_h(t[q].y));
+  }
+  unsigned char* stage = sh.stage[warp];
+#pragma unroll
+  for (int r = 0; r < RS_DOWN_ROWS; ++r, out += row_bytes) {
+    if (r >= nq) break;
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const float* za = z[2 * q] + r * SH::WZ;
+      const float* zb = z[2 * q + 1] + r * SH::WZ;
+      const f2 u = eval2<BMODE>(
+          cell2<BMODE>(make_float2(za[0], zb[0]), make_float2(za[1], zb[1]),
+                       make_float2(za[2], zb[2]), make_float2(za[3], zb[3]), eps, beta),
+          t[q], C0[q], h[q]);
+      // columns past the tile repeat its last and land after the row
+      rs_store<TOut>(stage, lane + 64 * q, u.x, a.out_dtype, a.clamp_float);
+      rs_store<TOut>(stage, lane + 64 * q + 32, u.y, a.out_dtype, a.clamp_float);
+    }
+    __syncwarp();
+    rs_flush<TOut>(out, a.out_sw, a.out_vec4, stage, nc, lane, a.out_dtype);
+    __syncwarp();
+  }
+}
+
+template <int BMODE, class TIn, class TOut, bool UP>
+__global__ void __launch_bounds__(RS_THREADS, 3)
+    resample_tiled_kernel(const __grid_constant__ ResampleArgs a, float eps, float beta) {
+  using SH = RsShared<UP>;
+  __shared__ SH sh;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int n = (int)a.n, m = (int)a.m;
+  const int tc = a.tile_cols, tr = RS_WARPS * a.warp_rows;
+  const int c0 = (int)blockIdx.x * tc, r0 = (int)blockIdx.y * tr;
+  const int64_t plane = blockIdx.z;
+  const int nc = min((int)a.m_out - c0, tc);
+  const int nr = min((int)a.n_out - r0, tr);
+  // every output column's and row's cell and offset; the first and last of
+  // them bound the input window
+  for (int c = tid; c < nc; c += RS_THREADS)
+    grid_pos(c0 + c, m, (int)a.m_out, a.div_x, sh.col_j[c], sh.col_t[c]);
+  if (tid < nr) {
+    float t;
+    grid_pos(r0 + tid, n, (int)a.n_out, a.div_y, sh.row_i[tid], t);
+    const float C0 = pos_c0(t), h = pos_h(t);
+    sh.row_a[tid] = make_float4(t, t, C0, C0);
+    sh.row_h[tid] = make_float2(h, h);
+  }
+  __syncthreads();
+  const int kfirst = sh.col_j[0] - 1, in_base = sh.row_i[0] - 1;
+  const int wc = sh.col_j[nc - 1] + 2 - kfirst + 1;  // <= RS_WC_UP, RS_WC_DOWN (host)
+  const int wr = sh.row_i[nr - 1] + 2 - in_base + 1; // <= RS_MAX_IN (host)
+  const int esz = elem_bytes<TIn>(a.in_dtype);
+  for (int r = tid; r < wr; r += RS_THREADS)
+    sh.in_off[r] = (int64_t)clamp_idx(in_base + r, n) * a.in_sh * esz;
+  if (UP) {
+    for (int c = tid; c < nc; c += RS_THREADS)
+      if (c == 0 || sh.col_j[c] != sh.col_j[c - 1]) sh.start[sh.col_j[c] - 1 - kfirst] = c;
+    if (tid == 0) sh.start[wc - 3] = nc;
+  }
+  __syncthreads();
+  const int q0 = warp * a.warp_rows;
+  const int nq = min(nr - q0, a.warp_rows);
+  if (nq <= 0) return;
+  const char* in_plane = static_cast<const char*>(a.in) + plane * a.in_sc * esz;
+  for (int k0 = 0; k0 < wc; k0 += 64)
+    column_pass<BMODE, TIn>(a, sh, warp, lane, q0, nq, in_base, kfirst, wc, k0, in_plane, esz, eps,
+                            beta);
+  __syncwarp();
+  const int osz = elem_bytes<TOut>(a.out_dtype);
+  char* out = static_cast<char*>(a.out) +
+              (plane * a.out_sc + (int64_t)(r0 + q0) * a.out_sh + (int64_t)c0 * a.out_sw) * osz;
+  const int64_t row_bytes = a.out_sh * osz;
+  if constexpr (UP) {
+    const int cells = wc - 3;
+    int most = 0;  // outputs of the fullest cell
+    for (int k = lane; k < cells; k += 32) most = max(most, sh.start[k + 1] - sh.start[k]);
+    most = __reduce_max_sync(0xffffffffu, most);
+    if (most <= 2)
+      row_pass_up<BMODE, TOut, 2>(a, sh, warp, lane, nq, nc, cells, most, out, row_bytes, eps, beta);
+    else if (most == 3)
+      row_pass_up<BMODE, TOut, 3>(a, sh, warp, lane, nq, nc, cells, most, out, row_bytes, eps, beta);
+    else
+      row_pass_up<BMODE, TOut, 4>(a, sh, warp, lane, nq, nc, cells, most, out, row_bytes, eps, beta);
+  } else {
+    row_pass_down<BMODE, TOut>(a, sh, warp, lane, nq, nc, kfirst, out, row_bytes, eps, beta);
+  }
+}
+
+template <int BMODE, class TIn, class TOut>
+cudaError_t launch_form(const ResampleArgs& a, float eps, float beta, cudaStream_t stream) {
+  if (!a.tiled) {
+    const dim3 block(32, 8);
+    const dim3 grid((unsigned)((a.m_out + 31) / 32), (unsigned)((a.n_out + 7) / 8),
+                    (unsigned)a.planes);
+    resample_kernel<BMODE, TIn, TOut><<<grid, block, 0, stream>>>(a, eps, beta);
+    return cudaGetLastError();
+  }
+  const int tr = RS_WARPS * a.warp_rows;
+  const dim3 grid((unsigned)((a.m_out + a.tile_cols - 1) / a.tile_cols),
+                  (unsigned)((a.n_out + tr - 1) / tr), (unsigned)a.planes);
+  if (a.up)
+    resample_tiled_kernel<BMODE, TIn, TOut, true><<<grid, RS_THREADS, 0, stream>>>(a, eps, beta);
+  else
+    resample_tiled_kernel<BMODE, TIn, TOut, false><<<grid, RS_THREADS, 0, stream>>>(a, eps, beta);
   return cudaGetLastError();
 }
 
 template <class TIn, class TOut>
-cudaError_t launch_tiled_beta(const ResampleArgs& a, float eps, float beta, int bmode,
+cudaError_t launch_beta(const ResampleArgs& a, float eps, float beta, int bmode,
                               cudaStream_t stream) {
   switch (bmode) {
-    case B2: return launch_tiled<B2, TIn, TOut>(a, eps, beta, stream);
-    case B2R: return launch_tiled<B2R, TIn, TOut>(a, eps, beta, stream);
-    case B0: return launch_tiled<B0, TIn, TOut>(a, eps, beta, stream);
-    default: return launch_tiled<BGEN, TIn, TOut>(a, eps, beta, stream);
+    case B2: return launch_form<B2, TIn, TOut>(a, eps, beta, stream);
+    case B2R: return launch_form<B2R, TIn, TOut>(a, eps, beta, stream);
+    case B0: return launch_form<B0, TIn, TOut>(a, eps, beta, stream);
+    default: return launch_form<BGEN, TIn, TOut>(a, eps, beta, stream);
   }
 }
 
 }  // namespace
+
+static int resample_sms() {
+  static std::atomic<int> known[64];
+  int dev = 0, v = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 152;
+  v = known[dev].load(std::memory_order_relaxed);
+  if (v > 0) return v;
+  if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 152;
+  known[dev].store(v, std::memory_order_relaxed);
+  return v;
+}
 
 static AxisDiv axis_div(int64_t n, int64_t n_out) {
   AxisDiv d{1u, 0, 0, 0, 0.f};
@@ -421,34 +582,40 @@ cudaError_t launch_resample(const ResampleArgs& a_in, float eps, float beta, int
   ResampleArgs a = a_in;
   a.div_y = axis_div(a.n, a.n_out);
   a.div_x = axis_div(a.m, a.m_out);
-  // the tiled form reads at most RS_WC window columns and sizes its window
-  // rows from the y ratio: spacing ratios (n - 1)/(n_out - 1) <= 2 per axis
-  const bool tiled = (a.m_out == 1 || 2 * (a.m_out - 1) >= (a.m - 1)) &&
-                     (a.n_out == 1 || 2 * (a.n_out - 1) >= (a.n - 1));
-  if (tiled) {
-    a.tile_rows = a.n_out >= a.n ? RS_TR_UP : RS_TR_DOWN;
-    a.win_rows =
-        (a.n_out > 1 ? (int)((int64_t)(a.tile_rows - 1) * (a.n - 1) / (a.n_out - 1)) : 0) + 5;
-    const int i = a.in_dtype, o = a.out_dtype;
-    if (i == DT_U8 && o == DT_U8) return launch_tiled_beta<uint8_t, uint8_t>(a, eps, beta, bmode, stream);
-    if (i == DT_F16 && o == DT_F16) return launch_tiled_beta<__half, __half>(a, eps, beta, bmode, stream);
-    if (i == DT_BF16 && o == DT_BF16)
-      return launch_tiled_beta<__nv_bfloat16, __nv_bfloat16>(a, eps, beta, bmode, stream);
-    if (i == DT_F32 && o == DT_F32) return launch_tiled_beta<float, float>(a, eps, beta, bmode, stream);
-    if (i == DT_U8 && o == DT_F32) return launch_tiled_beta<uint8_t, float>(a, eps, beta, bmode, stream);
-    if (i == DT_F32 && o == DT_U8) return launch_tiled_beta<float, uint8_t>(a, eps, beta, bmode, stream);
-    return launch_tiled_beta<Dyn, Dyn>(a, eps, beta, bmode, stream);
+  // spacing ratios (n - 1)/(n_out - 1) <= 2 per axis, and something to
+  // interpolate on both
+  a.tiled = a.n > 1 && a.m > 1 &&
+            (a.m_out == 1 || 2 * (a.m_out - 1) >= (a.m - 1)) &&
+            (a.n_out == 1 || 2 * (a.n_out - 1) >= (a.n - 1));
+  if (a.tiled) {
+    a.up = a.m_out >= a.m;
+    // magnified: as many columns as 64 window columns serve (a span of d input
+    // spacings touches at most ceil(d) + 4 samples), in whole words
+    int64_t tc = RS_TC_DOWN;
+    if (a.up) {
+      tc = (RS_WC_UP - 4) * (a.m_out - 1) / (a.m - 1) + 1;
+      tc = std::min<int64_t>(tc, RS_TC_MAX) & ~int64_t(3);
+    }
+    a.tile_cols = (int)tc;
+    // rows per warp: each warp loads 3 rows more than its cells, so more rows
+    // cost less, as long as about every SM gets a tile (reduced rows: three
+    // in four SMs; halving 4 rows there doubles the halo's share)
+    const int sms = resample_sms(), least = a.n_out >= a.n ? sms : 3 * sms / 4;
+    const int64_t strips = (a.m_out + tc - 1) / tc * a.planes;
+    int rows = a.n_out >= a.n && a.up ? RS_MAX_ROWS : RS_DOWN_ROWS;
+    while (rows > 1 && strips * ((a.n_out + RS_WARPS * rows - 1) / (RS_WARPS * rows)) < least)
+      rows >>= 1;
+    a.warp_rows = rows;
   }
-  const dim3 block(32, 8);
-  const dim3 grid((unsigned)((a.m_out + 31) / 32), (unsigned)((a.n_out + 7) / 8),
-                  (unsigned)a.planes);
-  switch (bmode) {
-    case B2: resample_kernel<B2><<<grid, block, 0, stream>>>(a, eps, beta); break;
-    case B2R: resample_kernel<B2R><<<grid, block, 0, stream>>>(a, eps, beta); break;
-    case B0: resample_kernel<B0><<<grid, block, 0, stream>>>(a, eps, beta); break;
-    default: resample_kernel<BGEN><<<grid, block, 0, stream>>>(a, eps, beta); break;
-  }
-  return cudaGetLastError();
+  const int i = a.in_dtype, o = a.out_dtype;
+  if (i == DT_U8 && o == DT_U8) return launch_beta<uint8_t, uint8_t>(a, eps, beta, bmode, stream);
+  if (i == DT_F16 && o == DT_F16) return launch_beta<__half, __half>(a, eps, beta, bmode, stream);
+  if (i == DT_BF16 && o == DT_BF16)
+    return launch_beta<__nv_bfloat16, __nv_bfloat16>(a, eps, beta, bmode, stream);
+  if (i == DT_F32 && o == DT_F32) return launch_beta<float, float>(a, eps, beta, bmode, stream);
+  if (i == DT_U8 && o == DT_F32) return launch_beta<uint8_t, float>(a, eps, beta, bmode, stream);
+  if (i == DT_F32 && o == DT_U8) return launch_beta<float, uint8_t>(a, eps, beta, bmode, stream);
+  return launch_beta<Dyn, Dyn>(a, eps, beta, bmode, stream);
 }
 
 }  // namespace wdweno

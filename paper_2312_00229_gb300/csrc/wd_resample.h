@@ -32,8 +32,11 @@ struct ResampleArgs {
   int clamp_float;
   int out_vec4;                  // unit column stride, rows and planes of 4-element
                                  // multiples, 4-element aligned base
-  int win_rows;                  // window rows of the tiled kernel (set by the launcher)
-  int tile_rows;                 // output rows per tile of the tiled kernel (launcher)
+  // set by the launcher
+  int tiled;                     // the separable tiled kernel serves the ratios
+  int up;                        // the columns are magnified
+  int tile_cols;                 // output columns per tile
+  int warp_rows;                 // output rows per warp
   AxisDiv div_y, div_x;          // division by n_out - 1, m_out - 1 (set by the launcher)
 };
 
