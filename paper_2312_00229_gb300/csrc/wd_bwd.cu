@@ -58,6 +58,10 @@
 // 74% and 65% busy,
 // 379 and 169 M warp instructions (455 and 233 before).
 #include "wd_bwd.h"
+
+#include <atomic>
+#include <cmath>
+
 #include "wd_packed.cuh"
 
 namespace wdweno {
@@ -924,93 +928,120 @@ __global__ void __launch_bounds__(NT2, NT2 == NT_NARROW ? 4 : 2)
   sweep_band(sw, &R.A[0][sw.u], s_begin, s_end, s_lo, s_hi);
 }
 
-// Rows per band: the band count that minimises waves x (rows + fill steps).
-int band_rows(int64_t rows_total, int64_t ctas_per_band_row, int fill, int resident) {
-  int best = (int)rows_total;
-  double best_cost = 1e300;
-  for (int bands = 1; bands <= 64; ++bands) {
-    const int64_t h = (rows_total + bands - 1) / bands;
-    if (h < 16 && bands > 1) break;
-    const int64_t ctas = ctas_per_band_row * bands;
-    const int64_t waves = (ctas + resident - 1) / resident;
-    const double cost = double(waves) * double(h + fill);
-    if (cost < best_cost - 1e-9) {
-      best_cost = cost;
-      best = (int)h;
+// Resident CTAs per SM of a kernel with `smem` bytes of dynamic shared memory,
+// which this also allows it: a function of the kernel and the device, asked
+// once per pair (the two queries took 6 us of host time a kernel and call).
+template <class K>
+cudaError_t resident_ctas(K kern, int threads, size_t smem, int dev, std::atomic<int>* known,
+                          int* occ) {
+  const int i = dev >= 0 && dev < 64 ? dev : -1;
+  *occ = i >= 0 ? known[i].load(std::memory_order_acquire) : 0;
+  if (*occ > 0) return cudaSuccess;
+  cudaError_t e =
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, kern, threads, smem);
+  if (e == cudaSuccess && i >= 0 && *occ > 0) known[i].store(*occ, std::memory_order_release);
+  return e;
+}
+
+// Time model of a sweep (as wd_fwd_model.h): a band of `rows` rows takes
+// rows + fill steps, and a step, with k CTAs on an SM,
+// sqrt(lat^2 + (k issue)^2) us.
+struct SweepModel {
+  float lat, issue[2];  // (narrow, wide)
+  float fill;
+};
+// The step times follow the full-size runs (1.1 and 0.49 us with the CTAs
+// resident), the others short bands on an idle GPU; latencies of 0.5 to 0.75
+// and 0.3 to 0.5 us and fills 25% off choose shapes within 2% of each other.
+// Bands of at least 16 rows, the rule before, left small images on a few CTAs:
+// 3x64x64 39.5 -> 23.0 us, 1x128x200 -> 23.6, 3x256x256 43.3 -> 40.5.
+constexpr SweepModel PLUS_MODEL = {0.50f, {0.31f, 0.46f}, 13.f};
+constexpr SweepModel CROSS_MODEL = {0.30f, {0.133f, 0.20f}, 10.f};
+
+struct SweepShape {
+  int wide, strips, rows;
+  int64_t bands;
+};
+
+// The CTA width and band height of least modelled time.
+SweepShape pick_shape(const SweepModel& model, const int (&occ)[2], const int (&tw)[2], int sms,
+                      int64_t rows_total, int64_t cols_total, int64_t planes) {
+  SweepShape best{0, 1, (int)rows_total, 1};
+  double best_us = 1e300;
+  for (int i = 0; i < 2; ++i) {
+    if (occ[i] < 1) continue;
+    const int64_t strips = (cols_total + tw[i] - 1) / tw[i], slots = (int64_t)occ[i] * sms;
+    auto step = [&](int64_t k) {
+      const double q = double(k) * model.issue[i];
+      return std::sqrt(double(model.lat) * model.lat + q * q);
+    };
+    const double full = step(occ[i]);
+    int64_t last = -1;
+    for (int64_t b = 1; b <= rows_total && b <= 65535; ++b) {
+      const int64_t rows = (rows_total + b - 1) / b;
+      if (rows == last) continue;
+      // bands below 16 rows only where they still find idle CTA slots
+      if (b > 1 && (rows < 2 || (rows < 16 && strips * planes * b > slots))) break;
+      last = rows;
+      const int64_t bands = (rows_total + rows - 1) / rows, ctas = strips * planes * bands;
+      const int64_t rest = ctas % slots;
+      double us = double(ctas / slots) * full;
+      if (rest) us += step((rest + sms - 1) / sms);
+      us *= double(rows) + model.fill;
+      if (us < best_us - 1e-9) {
+        best_us = us;
+        best = SweepShape{i, (int)strips, (int)rows, bands};
+      }
     }
   }
   return best;
 }
 
-// One sweep kernel with the CTA width, of NT_NARROW and NT_WIDE, that
-// spends the least: for each width, the band height band_rows chooses, then
-// the per-SM work ceil(CTAs / SMs) x threads x (rows per band + fill).
-struct SweepShape {
-  const void* fn;
-  size_t smem;
-  int threads, occ, strips, rows;
-  int64_t bands;
-};
-
-template <class KN, class KW>
-cudaError_t pick_shape(KN kn, KW kw, int roles, size_t smem_n, size_t smem_w, int tw_n, int tw_w,
-                       int64_t rows_total, int64_t cols_total, int64_t planes, int fill,
-                       SweepShape* best) {
-  int dev = 0, sms = 0;
-  cudaError_t e;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
-    return e;
-  const void* fns[2] = {(const void*)kn, (const void*)kw};
-  const size_t smems[2] = {smem_n, smem_w};
-  const int nts[2] = {NT_NARROW, NT_WIDE}, tws[2] = {tw_n, tw_w};
-  double best_cost = -1.0;
-  for (int i = 0; i < 2; ++i) {
-    if ((e = cudaFuncSetAttribute(fns[i], cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)smems[i])) != cudaSuccess)
-      return e;
-    int occ = 0;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fns[i], roles * nts[i], smems[i])) !=
-        cudaSuccess)
-      return e;
-    if (occ < 1) continue;
-    const int64_t strips = (cols_total + tws[i] - 1) / tws[i];
-    const int h = band_rows(rows_total, strips * planes, fill, occ * sms);
-    const int64_t bands = (rows_total + h - 1) / h;
-    const int64_t per_sm = (strips * bands * planes + sms - 1) / sms;
-    const double cost = double(per_sm) * nts[i] * double(h + fill);
-    if (best_cost < 0.0 || cost < best_cost) {
-      best_cost = cost;
-      *best = SweepShape{fns[i], smems[i], nts[i], occ, (int)strips, h, bands};
-    }
-  }
-  return best_cost < 0.0 ? cudaErrorInvalidConfiguration : cudaSuccess;
-}
-
 template <int BMODE>
 cudaError_t launch_all(const BwdArgs& a, const MethodConsts& k, cudaStream_t st) {
+  static std::atomic<int> known[4][64], known_sms[64];
+  constexpr size_t plus_n = sizeof(RingsPlus<NT_NARROW>), plus_w = sizeof(RingsPlus<NT_WIDE>);
+  constexpr size_t cross_n = sizeof(RingsCross<NT_NARROW>), cross_w = sizeof(RingsCross<NT_WIDE>);
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  int sms = dev >= 0 && dev < 64 ? known_sms[dev].load(std::memory_order_relaxed) : 0;
+  if (sms <= 0) {
+    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
+      return e;
+    if (dev >= 0 && dev < 64) known_sms[dev].store(sms, std::memory_order_relaxed);
+  }
+  int occ1[2], occ2[2];
+  if ((e = resident_ctas(k_bwd_plus<BMODE, NT_NARROW>, 2 * NT_NARROW, plus_n, dev, known[0],
+                         &occ1[0])) != cudaSuccess ||
+      (e = resident_ctas(k_bwd_plus<BMODE, NT_WIDE>, 2 * NT_WIDE, plus_w, dev, known[1],
+                         &occ1[1])) != cudaSuccess ||
+      (e = resident_ctas(k_bwd_cross<BMODE, NT_NARROW>, NT_NARROW, cross_n, dev, known[2],
+                         &occ2[0])) != cudaSuccess ||
+      (e = resident_ctas(k_bwd_cross<BMODE, NT_WIDE>, NT_WIDE, cross_w, dev, known[3],
+                         &occ2[1])) != cudaSuccess)
+    return e;
+  if ((occ1[0] < 1 && occ1[1] < 1) || (occ2[0] < 1 && occ2[1] < 1))
+    return cudaErrorInvalidConfiguration;
   // k_bwd_plus: the extended grid, rows and columns [-2, n+2) x [-2, m+2)
-  SweepShape s1, s2;
-  cudaError_t e = pick_shape(k_bwd_plus<BMODE, NT_NARROW>, k_bwd_plus<BMODE, NT_WIDE>, 2,
-                             sizeof(RingsPlus<NT_NARROW>), sizeof(RingsPlus<NT_WIDE>),
-                             NT_NARROW - HL1 - HR1, NT_WIDE - HL1 - HR1,
-                             a.n + 2 * BWD_GHOST, a.m + 2 * BWD_GHOST, a.planes, 10, &s1);
-  if (e != cudaSuccess) return e;
+  const SweepShape s1 =
+      pick_shape(PLUS_MODEL, occ1, {NT_NARROW - HL1 - HR1, NT_WIDE - HL1 - HR1}, sms,
+                 a.n + 2 * BWD_GHOST, a.m + 2 * BWD_GHOST, a.planes);
   const dim3 g1((unsigned)s1.strips, (unsigned)s1.bands, (unsigned)a.planes);
-  if (s1.threads == NT_WIDE)
-    k_bwd_plus<BMODE, NT_WIDE><<<g1, 2 * NT_WIDE, s1.smem, st>>>(a, k, s1.rows);
+  if (s1.wide)
+    k_bwd_plus<BMODE, NT_WIDE><<<g1, 2 * NT_WIDE, plus_w, st>>>(a, k, s1.rows);
   else
-    k_bwd_plus<BMODE, NT_NARROW><<<g1, 2 * NT_NARROW, s1.smem, st>>>(a, k, s1.rows);
+    k_bwd_plus<BMODE, NT_NARROW><<<g1, 2 * NT_NARROW, plus_n, st>>>(a, k, s1.rows);
   // k_bwd_cross: image rows and columns, ghosts folded at the edges
-  e = pick_shape(k_bwd_cross<BMODE, NT_NARROW>, k_bwd_cross<BMODE, NT_WIDE>, 1,
-                 sizeof(RingsCross<NT_NARROW>), sizeof(RingsCross<NT_WIDE>),
-                 NT_NARROW - HL2 - HR2, NT_WIDE - HL2 - HR2, a.n, a.m, a.planes, 8, &s2);
-  if (e != cudaSuccess) return e;
+  const SweepShape s2 = pick_shape(CROSS_MODEL, occ2, {NT_NARROW - HL2 - HR2, NT_WIDE - HL2 - HR2},
+                                   sms, a.n, a.m, a.planes);
   const dim3 g2((unsigned)s2.strips, (unsigned)s2.bands, (unsigned)a.planes);
-  if (s2.threads == NT_WIDE)
-    k_bwd_cross<BMODE, NT_WIDE><<<g2, NT_WIDE, s2.smem, st>>>(a, k, s2.rows);
+  if (s2.wide)
+    k_bwd_cross<BMODE, NT_WIDE><<<g2, NT_WIDE, cross_w, st>>>(a, k, s2.rows);
   else
-    k_bwd_cross<BMODE, NT_NARROW><<<g2, NT_NARROW, s2.smem, st>>>(a, k, s2.rows);
+    k_bwd_cross<BMODE, NT_NARROW><<<g2, NT_NARROW, cross_n, st>>>(a, k, s2.rows);
   return cudaGetLastError();
 }
 
