@@ -14,6 +14,7 @@ from typing import List, Optional, Sequence
 
 import torch
 
+from . import autotune
 from . import binding as B
 
 _DT = {torch.uint8: B.WENO_U8, torch.float16: B.WENO_F16, torch.bfloat16: B.WENO_BF16,
@@ -45,21 +46,34 @@ class Params:
     nbr_c: float = 0.125
 
     def c(self) -> B.weno_params:
-        p = B.weno_params()
-        p.beta, p.k_eps, p.h = float(self.beta), float(self.k_eps), float(self.h)
-        p.si_scale, p.out_mode, p.clamp_float = int(self.si_scale), int(self.out_mode), int(
-            bool(self.clamp_float))
-        p.data_bound = float(self.data_bound)
-        p.nbr_c = float(self.nbr_c)
-        return p
+        return B.weno_params(float(self.beta), float(self.k_eps), float(self.h),
+                             int(self.si_scale), int(self.out_mode), int(bool(self.clamp_float)),
+                             float(self.data_bound), float(self.nbr_c))
+
+
+_DEFAULT = Params()
+_DEFAULT_C = _DEFAULT.c()  # (the library only reads it)
+
+
+def _params_c(params: Params) -> B.weno_params:
+    return _DEFAULT_C if params is _DEFAULT else params.c()
+
+
+def _level_params(p: Params, lvl: int, bound: float, out_mode: int) -> Params:
+    """Parameters of level `lvl` of a chain: spacing h / 2^lvl, |input| <= bound."""
+    return Params(p.beta, p.k_eps, p.h / (1 << lvl), p.si_scale, out_mode, p.clamp_float, bound,
+                  p.nbr_c)
 
 
 def lib():
     return B.load()
 
 
-def _stream(device) -> ctypes.c_void_p:
-    return ctypes.c_void_p(torch.cuda.current_stream(device).cuda_stream)
+def _stream(device: torch.device) -> int:
+    """Raw handle of the current stream of a device."""
+    index = device.index
+    return torch._C._cuda_getCurrentRawStream(
+        torch.cuda.current_device() if index is None else index)
 
 
 def _require_cuda(t: torch.Tensor, name: str):
@@ -73,30 +87,26 @@ def _planes(t: torch.Tensor, layout: str):
     """(height, width, channels, stride_c, stride_h, stride_w) of a tensor,
     folding a leading batch dimension into the channel count when the planes
     are uniformly strided."""
-    if t.dim() == 2:
-        return t.shape[0], t.shape[1], 1, 1, t.stride(0), t.stride(1)
+    shape, st, dim = t.shape, t.stride(), t.dim()
+    if dim == 2:
+        return shape[0], shape[1], 1, 1, st[0], st[1]
     if layout == "hwc":
-        if t.dim() != 3:
+        if dim != 3:
             raise ValueError("hwc layout needs a 3-D tensor [H, W, C]")
-        return t.shape[0], t.shape[1], t.shape[2], t.stride(2), t.stride(0), t.stride(1)
-    if t.dim() == 3:
-        return t.shape[1], t.shape[2], t.shape[0], t.stride(0), t.stride(1), t.stride(2)
-    if t.dim() == 4:
-        N, C = t.shape[0], t.shape[1]
-        if N == 1 or C == 1 or t.stride(0) == C * t.stride(1):
-            sc = t.stride(1) if C > 1 else t.stride(0)
-            return t.shape[2], t.shape[3], N * C, max(sc, 1), t.stride(2), t.stride(3)
+        return shape[0], shape[1], shape[2], st[2], st[0], st[1]
+    if dim == 3:
+        return shape[1], shape[2], shape[0], st[0], st[1], st[2]
+    if dim == 4:
+        N, C = shape[0], shape[1]
+        if N == 1 or C == 1 or st[0] == C * st[1]:
+            return shape[2], shape[3], N * C, max(st[1] if C > 1 else st[0], 1), st[2], st[3]
         raise ValueError("4-D input needs uniformly strided planes (e.g. contiguous NCHW)")
     raise ValueError("expected a 2-D, 3-D or 4-D tensor")
 
 
 def image(t: torch.Tensor, layout: str = "chw") -> B.weno_image:
     h, w, c, sc, sh, sw = _planes(t, layout)
-    im = B.weno_image()
-    im.data = t.data_ptr()
-    im.height, im.width, im.channels = int(h), int(w), int(c)
-    im.stride_c, im.stride_h, im.stride_w = int(max(sc, 1)), int(max(sh, 1)), int(max(sw, 1))
-    return im
+    return B.weno_image(t.data_ptr(), h, w, c, max(sc, 1), max(sh, 1), max(sw, 1))
 
 
 def out_hw(h: int, w: int, params: Params):
@@ -106,10 +116,9 @@ def out_hw(h: int, w: int, params: Params):
 
 def _out_like(x: torch.Tensor, params: Params, layout: str, dtype) -> torch.Tensor:
     shape = list(x.shape)
-    if layout == "hwc":
-        shape[0], shape[1] = out_hw(shape[0], shape[1], params)
-    else:
-        shape[-2], shape[-1] = out_hw(shape[-2], shape[-1], params)
+    d = 1 if params.out_mode == B.WENO_OUT_2N_MINUS_1 else 0
+    r = 0 if layout == "hwc" else -2
+    shape[r], shape[r + 1] = 2 * shape[r] - d, 2 * shape[r + 1] - d
     return torch.empty(shape, dtype=dtype, device=x.device)
 
 
@@ -119,11 +128,16 @@ def _level_out(x: torch.Tensor, params: Params, layout: str, dtype) -> torch.Ten
     level reads it, and rows that all start on a four-element boundary are
     written with one vector store per thread and fine row (odd widths of the
     2n-1 grid otherwise take three)."""
-    if layout == "hwc" or x.dim() < 2:
-        return _out_like(x, params, layout, dtype)
     h, w = out_hw(x.shape[-2], x.shape[-1], params)
-    return torch.empty((*x.shape[:-2], h, (w + 3) // 4 * 4), dtype=dtype,
-                       device=x.device)[..., :w]
+    if layout == "hwc" or w % 4 == 0:
+        return _out_like(x, params, layout, dtype)
+    ld = (w + 3) // 4 * 4
+    strides, size = [1, ld], h * ld
+    for n in reversed(x.shape[:-2]):
+        strides.append(size)
+        size *= n
+    return torch.empty_strided((*x.shape[:-2], h, w), strides[:0:-1] + [1], dtype=dtype,
+                               device=x.device)
 
 
 def zoom2x_fwd(x: torch.Tensor, params: Optional[Params] = None, out_dtype=None,
@@ -135,7 +149,7 @@ def zoom2x_fwd(x: torch.Tensor, params: Optional[Params] = None, out_dtype=None,
     choice for this size class (see ``autotune``), 0 = the library default.
     ``tile_width``: output columns per CTA, 247 (256 threads) or 119 (128
     threads); 0 = the library's choice for the image width."""
-    params = params or Params()
+    params = params or _DEFAULT
     _require_cuda(x, "x")
     if x.numel() == 0:
         raise ValueError("empty input")
@@ -143,12 +157,10 @@ def zoom2x_fwd(x: torch.Tensor, params: Optional[Params] = None, out_dtype=None,
         out = _out_like(x, params, layout, out_dtype or x.dtype)
     _require_cuda(out, "out")
     if rows_per_tile is None:
-        from . import autotune
-        rows_per_tile = autotune.lookup(x, out.dtype, layout)
-        if tile_width == 0:
-            tile_width = autotune.lookup_width(x, out.dtype, layout)
+        rows_per_tile, width = autotune.lookup_shape(x, out.dtype, layout)
+        tile_width = tile_width or width
     rc = B.weno_zoom2x_fwd_tiled(image(x, layout), _DT[x.dtype], image(out, layout),
-                                 _DT[out.dtype], params.c(), rows_per_tile, int(tile_width),
+                                 _DT[out.dtype], _params_c(params), rows_per_tile, tile_width,
                                  _stream(x.device))
     B.check("weno_zoom2x_fwd", rc)
     return out
@@ -157,7 +169,7 @@ def zoom2x_fwd(x: torch.Tensor, params: Optional[Params] = None, out_dtype=None,
 def zoom2x_bwd(x: torch.Tensor, grad_out: torch.Tensor, params: Optional[Params] = None,
                layout: str = "chw", workspace: Optional[torch.Tensor] = None) -> torch.Tensor:
     """Input gradient of the zoom for FP32 data (``weno_zoom2x_bwd``)."""
-    params = params or Params()
+    params = params or _DEFAULT
     _require_cuda(x, "x")
     _require_cuda(grad_out, "grad_out")
     if x.dtype != torch.float32 or grad_out.dtype != torch.float32:
@@ -167,7 +179,7 @@ def zoom2x_bwd(x: torch.Tensor, grad_out: torch.Tensor, params: Optional[Params]
     need = B.weno_zoom2x_bwd_workspace_bytes(xi)
     if workspace is None or workspace.numel() < need:
         workspace = torch.empty(need, dtype=torch.uint8, device=x.device)
-    rc = B.weno_zoom2x_bwd(xi, image(grad_out, layout), image(grad_in, layout), params.c(),
+    rc = B.weno_zoom2x_bwd(xi, image(grad_out, layout), image(grad_in, layout), _params_c(params),
                            ctypes.c_void_p(workspace.data_ptr()), need, _stream(x.device))
     B.check("weno_zoom2x_bwd", rc)
     return grad_in
@@ -192,7 +204,7 @@ class WenoZoom2x(torch.autograd.Function):
 def zoom2x(x: torch.Tensor, params: Optional[Params] = None, out_dtype=None,
            layout: str = "chw") -> torch.Tensor:
     """2x zoom; differentiable for FP32 inputs that require grad."""
-    params = params or Params()
+    params = params or _DEFAULT
     if torch.is_grad_enabled() and x.requires_grad:
         if x.dtype != torch.float32 or (out_dtype not in (None, torch.float32)):
             raise TypeError("gradients are supported for FP32 in and out")
@@ -231,7 +243,7 @@ def cascade_zoom(x: torch.Tensor, levels: int, params: Optional[Params] = None, 
     ``fused=True`` runs every level in one persistent launch
     (``weno_zoom2x_cascade``; FP32 intermediates in a workspace) with the
     same result."""
-    params = params or Params()
+    params = params or _DEFAULT
     if fused:
         if inter_dtype != torch.float32:
             raise ValueError("the fused cascade keeps FP32 intermediates")
@@ -247,7 +259,7 @@ def cascade_zoom(x: torch.Tensor, levels: int, params: Optional[Params] = None, 
         else:
             shape[-2], shape[-1] = oh, ow
         out = torch.empty(shape, dtype=out_dtype or x.dtype, device=x.device)
-        xi, oi, pc = image(x, layout), image(out, layout), params.c()
+        xi, oi, pc = image(x, layout), image(out, layout), _params_c(params)
         nbytes = B.weno_zoom2x_cascade_workspace_bytes(xi, levels, pc)
         if nbytes == 0:
             raise ValueError("malformed cascade request")
@@ -261,7 +273,7 @@ def cascade_zoom(x: torch.Tensor, levels: int, params: Optional[Params] = None, 
     cur = x
     for lvl in range(levels):
         last = lvl == levels - 1
-        p = dataclasses.replace(params, h=params.h / (1 << lvl), data_bound=bounds[lvl])
+        p = _level_params(params, lvl, bounds[lvl], params.out_mode)
         if last:
             cur = zoom2x_fwd(cur, p, out_dtype=out_dtype or x.dtype, layout=layout)
         else:
@@ -281,7 +293,7 @@ def resample(x: torch.Tensor, out_h: int, out_w: int, params: Optional[Params] =
     ``out_h x out_w`` on endpoint-aligned grids (``weno_resample``).
     ``params.h`` is the spacing of the input grid; ``out_mode`` and
     ``si_scale`` do not apply."""
-    params = params or Params()
+    params = params or _DEFAULT
     _require_cuda(x, "x")
     if x.numel() == 0 or out_h < 1 or out_w < 1:
         raise ValueError("empty input or output")
@@ -294,7 +306,7 @@ def resample(x: torch.Tensor, out_h: int, out_w: int, params: Optional[Params] =
         out = torch.empty(shape, dtype=out_dtype or x.dtype, device=x.device)
     _require_cuda(out, "out")
     rc = B.weno_resample(image(x, layout), _DT[x.dtype], image(out, layout), _DT[out.dtype],
-                         params.c(), _stream(x.device))
+                         _params_c(params), _stream(x.device))
     B.check("weno_resample", rc)
     return out
 
@@ -314,18 +326,15 @@ def zoom_to(x: torch.Tensor, out_h: int, out_w: int, params: Optional[Params] = 
     (2n-1) grid up to the first size that covers the target, then tensor
     WENO resampling down to ``out_h x out_w`` (the 3x example zooms n to
     4n-3, then resamples to 3n)."""
-    params = params or Params()
+    params = params or _DEFAULT
     n, m = _hw(x, layout)
     k = zoom_levels(n, m, out_h, out_w)
     bounds = _level_bounds(x, params, k)
     cur = x
-    p = dataclasses.replace(params, out_mode=B.WENO_OUT_2N_MINUS_1)
     for lvl in range(k):
-        cur = zoom2x_fwd(cur, dataclasses.replace(p, h=params.h / (1 << lvl),
-                                                  data_bound=bounds[lvl]),
-                         layout=layout, out=_level_out(cur, p, layout, inter_dtype))
-    return resample(cur, out_h, out_w,
-                    dataclasses.replace(params, h=params.h / (1 << k), data_bound=bounds[k]),
+        p = _level_params(params, lvl, bounds[lvl], B.WENO_OUT_2N_MINUS_1)
+        cur = zoom2x_fwd(cur, p, layout=layout, out=_level_out(cur, p, layout, inter_dtype))
+    return resample(cur, out_h, out_w, _level_params(params, k, bounds[k], params.out_mode),
                     out_dtype=out_dtype or x.dtype, layout=layout)
 
 
@@ -339,7 +348,7 @@ class BatchedPlan:
                  outputs: Optional[Sequence[torch.Tensor]] = None, tile_width: int = 0):
         if len(images) == 0:
             raise ValueError("empty batch")
-        self.params = params or Params()
+        self.params = params or _DEFAULT
         self.layout = layout
         self.rows_per_tile = int(rows_per_tile)
         self.tile_width = int(tile_width)  # 0 = the library's default, 118
@@ -369,7 +378,7 @@ class BatchedPlan:
     def run(self) -> List[torch.Tensor]:
         rc = B.weno_zoom2x_batched(self.count, ctypes.c_void_p(self.d_in.data_ptr()), self.in_t,
                                    ctypes.c_void_p(self.d_out.data_ptr()), self.out_t,
-                                   self.params.c(), ctypes.c_void_p(self.workspace.data_ptr()),
+                                   _params_c(self.params), ctypes.c_void_p(self.workspace.data_ptr()),
                                    self.ws_bytes, self.rows_per_tile, self.tile_width,
                                    _stream(self.device))
         B.check("weno_zoom2x_batched", rc)
@@ -381,7 +390,6 @@ def zoom2x_batched(images: Sequence[torch.Tensor], params: Optional[Params] = No
     """Zooms images of independent sizes in one persistent launch."""
     tile_width = 0
     if rows_per_tile is None:
-        from . import autotune
         rows_per_tile, tile_width = autotune.lookup_batched(images, out_dtype, layout)
     return BatchedPlan(images, params, out_dtype, layout, rows_per_tile,
                        tile_width=tile_width).run()
@@ -404,7 +412,7 @@ class HostPipeline:
 
     def __init__(self, in_shape, in_dtype, params: Optional[Params] = None, out_dtype=None,
                  layout: str = "chw", device="cuda", depth: int = 3):
-        self.params = params or Params()
+        self.params = params or _DEFAULT
         self.layout = layout
         self.device = torch.device(device)
         self.depth = int(depth)

@@ -62,6 +62,9 @@ def size_class(x: torch.Tensor, out_dtype, layout: str) -> str:
 
 def _load() -> Dict[str, int]:
     global _cache
+    cache = _cache
+    if cache is not None:
+        return cache
     with _lock:
         if _cache is None:
             try:
@@ -84,6 +87,15 @@ def _save() -> None:
 def lookup(x: torch.Tensor, out_dtype, layout: str) -> int:
     """Cached band height for this size class, or 0 (library default)."""
     return _load().get(size_class(x, out_dtype, layout), 0)
+
+
+def lookup_shape(x: torch.Tensor, out_dtype, layout: str) -> Tuple[int, int]:
+    """Cached (band height, tile width) for this size class, or (0, 0)."""
+    cache = _load()
+    if not cache:
+        return 0, 0
+    key = size_class(x, out_dtype, layout)
+    return cache.get(key, 0), cache.get(key + "|tile_width", 0)
 
 
 def lookup_width(x: torch.Tensor, out_dtype, layout: str) -> int:

@@ -102,6 +102,8 @@ def lib_path() -> str:
 def load(build_if_missing: bool = True):
     """Loads (building first if needed) and returns the CDLL."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is None:
             path = _build.LIB
