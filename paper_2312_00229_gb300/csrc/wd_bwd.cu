@@ -53,10 +53,12 @@
 // 32x3x512x512, both kernels: 1078 us with the four-row rings and register
 // prefetch; 1001 with the row-pair sums, own-column registers and kept
 // stencils; 883 with the asynchronous copies; 856 with a forward and a
-// backward thread per column in k_bwd_plus (2x3x1024x1024: 276, 248, 238;
-// 3x256x256: 49, 45, 44).  Now 143 and 56 wavefronts a warp's step, LSU pipe
-// 74% and 65% busy,
-// 379 and 169 M warp instructions (455 and 233 before).
+// backward thread per column in k_bwd_plus; 816 with the forward threads also
+// requesting the gradients that the backward threads use, and strides read
+// from the constant bank (2x3x1024x1024: 276, 248, 238, 233; 3x256x256: 49, 45, 44,
+// 36, the last with the shapes of pick_shape).  Now 140 and 56 wavefronts a
+// warp's step, LSU pipe 78% and 63% busy, 377 and 176 M warp instructions
+// (455 and 233 before).  Two to five CTAs per SM in k_bwd_cross measure the same.
 #include "wd_bwd.h"
 
 #include <atomic>
@@ -117,7 +119,7 @@ struct RingsPlus {
   float4 DE[2][NT], DS[2][NT];
   float2 EZ[4][NT], SZ[4][NT], EG[4][NT], SG[4][NT];
   float EM[4][NT], SM[4][NT];
-  // Output gradients requested by the backward thread: fine rows 2r, columns
+  // Output gradients: fine rows 2r, columns
   // 2c, 2c + 1 (samples, E points), and 2r + 1 (S, x points)
   float2 GE[4][NT], GS[4][NT];
 };
@@ -386,11 +388,14 @@ template <int BMODE, int NT1>
 struct PlusForward {
   static constexpr int W = RingsPlus<NT1>::W;
   RingsPlus<NT1>& R;
-  const MethodConsts k;
-  float w;
+  const BwdArgs& a;       // (kernel parameters: read from the constant bank)
+  const MethodConsts& k;
   int t, u, n, a0, a1;
   const float* xin;  // input row s + 2 (clamped) of the column, in step s
-  int64_t x_sh;
+  // output gradients of the fine columns 2c (samples, S points) and 2c + 1
+  // (E and x points), which the column's backward thread reads
+  const float* gp;       // fine row 2 (s - 3), column 2c, in step s
+  bool g_pair, g_one0, g_one1;  // both columns inside and one aligned pair; else each
   // carried from step to step
   float4 six1, six2;          // phase-1 indicators of rows s-4, s-5
   float4 xs;                  // x stencils of row s-4: second differences
@@ -400,25 +405,51 @@ struct PlusForward {
   float sxv, sav;             // column second differences centred at X(s-6), A(s-5)
   float4 sie1, sis1;          // "+" indicators of row s-6
 
-  __device__ __forceinline__ PlusForward(RingsPlus<NT1>& R_, const BwdArgs& a,
+  __device__ __forceinline__ PlusForward(RingsPlus<NT1>& R_, const BwdArgs& a_,
                                          const MethodConsts& k_, int thread, int c, int a0_,
                                          int a1_)
-      : R(R_), k(k_), t(thread), u(thread + PAD), n((int)a.n), a0(a0_), a1(a1_) {
-    w = k.w;
-    x_sh = a.x_sh;
+      : R(R_), a(a_), k(k_), t(thread), u(thread + PAD), n((int)a_.n), a0(a0_), a1(a1_) {
     // the first request is that of step a0 - 6 - (AHEAD + 1)
     xin = a.x + (int64_t)blockIdx.z * a.x_sc + (int64_t)clampi(c, 0, (int)a.m - 1) * a.x_sw +
-          (int64_t)clampi(a0 - 6 - (AHEAD + 1) + 2, 0, n - 1) * x_sh;
+          (int64_t)clampi(a0 - 6 - (AHEAD + 1) + 2, 0, n - 1) * a.x_sh;
+    const int64_t Q = 2 * (int64_t)c;
+    const bool inside = Q >= 0 && Q < a.ocols;
+    g_pair = a.g_vec && inside && Q + 1 < a.ocols;
+    g_one0 = inside && !g_pair;
+    g_one1 = inside && Q + 1 < a.ocols && !g_pair;
+    const int s0 = a0 - 6;  // first step (requests start AHEAD + 1 steps before it)
+    gp = a.gout + (int64_t)blockIdx.z * a.g_sc + (inside ? Q : 0) * a.g_sw +
+         2 * (int64_t)(s0 - (AHEAD + 1) - 3) * a.g_sh;
     six1 = six2 = xs = sie1 = sis1 = zero4();
     xM0 = xM1 = x1 = x2 = ac1 = sxv = sav = 0.f;
   }
 
-  // Step s's request: input row s + 2 (to the ring; first read in step s + 3).
+  // Requests columns 2c, 2c + 1 of output-gradient row `row`, at q (FULL steps
+  // request rows known to lie inside the output; columns outside it stay zero
+  // from the rings' start).
+  template <bool FULL>
+  __device__ __forceinline__ void request_grad(float2* dst, const float* q, int row) const {
+    if (!FULL && (row < 0 || row >= (int)a.orows)) {
+      *dst = make_float2(0.f, 0.f);
+      return;
+    }
+    if (g_pair) copy_async<8>(dst, q);
+    if (g_one0) {
+      copy_async<4>(&dst->x, q);
+      if (g_one1) copy_async<4>(&dst->y, q + a.g_sw);
+    }
+  }
+
+  // Step s's requests: input row s + 2 (to the ring; first read in step
+  // s + 3) and the output gradients that step s + 3 uses.
   template <bool FULL, class SL>
   __device__ __forceinline__ void request(const int s, const SL& sl) {
     copy_async<4>(sl.template a<-2>(), xin);
-    if (s + 2 >= 0 && s + 2 < n - 1) xin += x_sh;
+    if (s + 2 >= 0 && s + 2 < n - 1) xin += a.x_sh;
+    request_grad<FULL>(&R.GE[sl.template m4<3>()][t], gp, 2 * (s - 3));
+    request_grad<FULL>(&R.GS[sl.template m4<4>()][t], gp - a.g_sh, 2 * (s - 4) + 1);
     copy_commit();
+    gp += 2 * a.g_sh;
   }
 
   // Each stage runs only on the rows the band's outputs need (the guards are
@@ -444,7 +475,7 @@ struct PlusForward {
     float x0 = 0.f;
     if (FULL || (s - 4 >= a0 - 4 && s - 4 <= a1 + 3)) {
       const float4 l = R.SIX[sl.template m2<4>()][u - 1], r = R.SIX[sl.template m2<4>()][u + 1];
-      const float4 D = fma4(w, add4(add4(six2, six), add4(l, r)), six1);
+      const float4 D = fma4(k.w, add4(add4(six2, six), add4(l, r)), six1);
       x0 = blend<BMODE>(D, xM0, xM1, xs, k.beta);
       R.X[sl.template m2<4>()][u] = x0;
     }
@@ -482,8 +513,8 @@ struct PlusForward {
       const float4 vs = add4(sis1, sis), ve = add4(sie1, sie);
       R.VS[sl.template m2<5>()][u] = vs;
       R.VE[sl.template m2<5>()][u] = ve;
-      R.DE[sl.template m2<5>()][t] = fma4(w, vs, sie);
-      R.DS[sl.template m2<5>()][t] = fma4(w, ve, sis1);
+      R.DE[sl.template m2<5>()][t] = fma4(k.w, vs, sie);
+      R.DS[sl.template m2<5>()][t] = fma4(k.w, ve, sis1);
       sie1 = sie; sis1 = sis;
       sxv = sxn; sav = san;
     }
@@ -496,82 +527,37 @@ template <int BMODE, int NT1>
 struct PlusBackward {
   static constexpr int W = RingsPlus<NT1>::W;
   RingsPlus<NT1>& R;
-  float w, k2, beta;
+  const BwdArgs& a;       // (kernel parameters: read from the constant bank)
+  const MethodConsts& k;
+  float k2;
   int t, u, a0, a1;
   float* wxb;            // X_bar row s - 10 of the column
-  int64_t ws_ld, ws_ab;  // workspace row stride; from X_bar row s-10 to A_bar row s-9
   bool col_out;
-  // output gradients of the fine columns 2c (samples, S points) and 2c + 1
-  // (E and x points)
-  const float* gp;       // fine row 2 (s - 3), column 2c, in step s
-  int64_t g_sh, g_sw;
-  int orows;
-  bool g_pair, g_one0, g_one1;  // both columns inside and one aligned pair; else each
   // carried from step to step
   float4 pe1, pe2, ps1;       // p_bar of E rows s-7, s-8 and of S row s-8
   float4 de1, ds1;            // 2 D_bar of E row s-7, S row s-8
   float4 sbE, sbS;            // own-column part of 2 SI_bar of E, S row s-8
   float xacc[4], aacc[4];     // X_bar rows s-10 .. s-7 and A_bar rows s-9 .. s-6
 
-  __device__ __forceinline__ PlusBackward(RingsPlus<NT1>& R_, const BwdArgs& a,
-                                          const MethodConsts& k, int thread, int c, int b0,
+  __device__ __forceinline__ PlusBackward(RingsPlus<NT1>& R_, const BwdArgs& a_,
+                                          const MethodConsts& k_, int thread, int c, int b0,
                                           int b1, int a0_, int a1_)
-      : R(R_), w(k.w), k2(k.kappa2 * k.kappa2), beta(k.beta), t(thread), u(thread + PAD),
-        a0(a0_), a1(a1_) {
-    const int64_t plane = blockIdx.z;
+      : R(R_), a(a_), k(k_), k2(k_.kappa2 * k_.kappa2), t(thread), u(thread + PAD), a0(a0_),
+        a1(a1_) {
     col_out = c >= b0 && c < b1;
-    const int64_t Q = 2 * (int64_t)c;
-    const bool inside = Q >= 0 && Q < a.ocols;
-    g_pair = a.g_vec && inside && Q + 1 < a.ocols;
-    g_one0 = inside && !g_pair;
-    g_one1 = inside && Q + 1 < a.ocols && !g_pair;
-    g_sh = a.g_sh;
-    g_sw = a.g_sw;
-    orows = (int)a.orows;
-    const int s0 = a0 - 6;  // first step (requests start AHEAD + 1 steps before it)
-    gp = a.gout + plane * a.g_sc + (inside ? Q : 0) * a.g_sw +
-         2 * (int64_t)(s0 - (AHEAD + 1) - 3) * g_sh;
-    ws_ld = a.m + 2 * BWD_GHOST;
-    const int64_t cells = (a.n + 2 * BWD_GHOST) * ws_ld;
-    ws_ab = cells + ws_ld;
-    wxb = a.ws + plane * 2 * cells + (int64_t)(s0 - 10 + BWD_GHOST) * ws_ld + (c + BWD_GHOST);
+    const int s0 = a0 - 6;  // first step
+    wxb = a.ws + (int64_t)blockIdx.z * 2 * a.ws_cells +
+          (int64_t)(s0 - 10 + BWD_GHOST) * a.ws_ld + (c + BWD_GHOST);
     pe1 = pe2 = ps1 = de1 = ds1 = sbE = sbS = zero4();
 #pragma unroll
     for (int j = 0; j < 4; ++j) xacc[j] = aacc[j] = 0.f;
-  }
-
-  // Requests columns 2c, 2c + 1 of output-gradient row `row`, at q (FULL steps
-  // request rows known to lie inside the output; columns outside it stay zero
-  // from the rings' start).
-  template <bool FULL>
-  __device__ __forceinline__ void request_grad(float2* dst, const float* q, int row) const {
-    if (!FULL && (row < 0 || row >= orows)) {
-      *dst = make_float2(0.f, 0.f);
-      return;
-    }
-    if (g_pair) copy_async<8>(dst, q);
-    if (g_one0) {
-      copy_async<4>(&dst->x, q);
-      if (g_one1) copy_async<4>(&dst->y, q + g_sw);
-    }
-  }
-
-  // Step s's requests: the output gradients that step s + 3 uses.
-  template <bool FULL, class SL>
-  __device__ __forceinline__ void request(const int s, const SL& sl) {
-    request_grad<FULL>(&R.GE[sl.template m4<3>()][t], gp, 2 * (s - 3));
-    request_grad<FULL>(&R.GS[sl.template m4<4>()][t], gp - g_sh, 2 * (s - 4) + 1);
-    copy_commit();
-    gp += 2 * g_sh;
   }
 
   // Guarded steps skip the work of points whose incoming adjoints are all
   // zero (a sparse output gradient); FULL steps do it, with the same result.
   template <bool FULL, class SL>
   __device__ __forceinline__ void step(const int s, const SL& sl) {
-    copy_wait<AHEAD>();
     sync_cta();
-    request<FULL>(s, sl);
     const float2 gE = R.GE[sl.template m4<6>()][t], gS = R.GS[sl.template m4<7>()][t];
     // the accumulators' newest rows start from the output gradient there
     aacc[3] = gE.x;  // sample (s-6, c)
@@ -587,7 +573,7 @@ struct PlusBackward {
     if (FULL || (s - 8 >= a0 - 2 && s - 8 <= a1 + 1)) {
       {
         // E(r,c) is read by S(r,c), S(r,c+1), S(r-1,c), S(r-1,c+1)
-        const float4 sb = fma4(w, R.VDS[sl.template m2<8>()][u + 1], sbE);
+        const float4 sb = fma4(k.w, R.VDS[sl.template m2<8>()][u + 1], sbE);
         float eh[3] = {0.f, 0.f, 0.f};
         if (FULL || any_nonzero(pe2, sb)) {
           const float* y = R.EY[sl.template m4<8>()] + u;
@@ -605,7 +591,7 @@ struct PlusBackward {
       }
       {
         // S(r,c) is read by E(r,c), E(r+1,c), E(r,c-1), E(r+1,c-1)
-        const float4 sb = fma4(w, R.VDE[sl.template m2<7>()][u - 1], sbS);
+        const float4 sb = fma4(k.w, R.VDE[sl.template m2<7>()][u - 1], sbS);
         float sh[3] = {0.f, 0.f, 0.f};
         if (FULL || any_nonzero(ps1, sb)) {
           const float* y = R.SY[sl.template m4<8>()] + u;
@@ -624,8 +610,8 @@ struct PlusBackward {
     }
     // ---- X_bar of row s-10 and the partial A_bar of row s-9 are complete ----
     if (col_out && (FULL || (s - 10 >= a0 && s - 10 < a1))) *wxb = xacc[0];
-    if (col_out && (FULL || (s - 9 >= a0 && s - 9 < a1))) wxb[ws_ab] = aacc[0];
-    wxb += ws_ld;
+    if (col_out && (FULL || (s - 9 >= a0 && s - 9 < a1))) wxb[a.ws_cells + a.ws_ld] = aacc[0];
+    wxb += a.ws_ld;  // (A_bar row s-9 lies ws_cells + ws_ld behind X_bar row s-10)
     xacc[0] = xacc[1]; xacc[1] = xacc[2]; xacc[2] = xacc[3];
     aacc[0] = aacc[1]; aacc[1] = aacc[2]; aacc[2] = aacc[3];
 
@@ -635,41 +621,31 @@ struct PlusBackward {
       if (FULL || (s - 6 <= a1 + 1 && gE.y != 0.f)) {
         // E(r,c): D reads S at (r-1,c), (r,c), (r-1,c+1), (r,c+1)
         const float4 D =
-            fma4(w, R.VS[sl.template m2<6>()][u + 1], R.DE[sl.template m2<6>()][t]);
+            fma4(k.w, R.VS[sl.template m2<6>()][u + 1], R.DE[sl.template m2<6>()][t]);
         const float* y = R.EY[sl.template m4<6>()] + u;
         const float2 z = R.EZ[sl.template m4<6>()][t];
         point_adjoint<BMODE>(make_float4(y[1], y[0], z.x, z.y), R.EM[sl.template m4<6>()][t], D,
-                             beta, gE.y, pe0, de);
+                             k.beta, gE.y, pe0, de);
       }
       if (FULL || (s - 7 >= a0 - 2 && s - 7 <= a1 + 1 && gS.x != 0.f)) {
         // S(r,c): D reads E at (r,c-1), (r,c), (r+1,c-1), (r+1,c)
         const float4 D =
-            fma4(w, R.VE[sl.template m2<6>()][u - 1], R.DS[sl.template m2<6>()][t]);
+            fma4(k.w, R.VE[sl.template m2<6>()][u - 1], R.DS[sl.template m2<6>()][t]);
         const float* y = R.SY[sl.template m4<7>()] + u;
         const float2 z = R.SZ[sl.template m4<7>()][t];
         point_adjoint<BMODE>(make_float4(y[0], y[-1], z.x, z.y), R.SM[sl.template m4<7>()][t], D,
-                             beta, gS.x, ps0, ds);
+                             k.beta, gS.x, ps0, ds);
       }
       const float4 vde = add4(de1, de), vds = add4(ds1, ds);  // rows s-7, s-6; s-8, s-7
       R.VDE[sl.template m2<6>()][u] = vde;
       R.VDS[sl.template m2<7>()][u] = vds;
-      sbE = fma4(w, vds, de1);
-      sbS = fma4(w, vde, ds);
+      sbE = fma4(k.w, vds, de1);
+      sbS = fma4(k.w, vde, ds);
       de1 = de; ds1 = ds;
       pe2 = pe1; pe1 = pe0; ps1 = ps0;
     }
   }
 };
-
-// Requests of the steps before the first, then the band's steps.
-template <class SW>
-__device__ __forceinline__ void run_role(SW& sw, float* ringA, int s_begin, int s_end, int s_lo,
-                                         int s_hi) {
-#pragma unroll 1
-  for (int s = s_begin - (AHEAD + 1); s < s_begin; ++s)
-    sw.template request<false>(s, RowsRT<SW::W>{ringA, s});
-  sweep_band(sw, ringA, s_begin, s_end, s_lo, s_hi);
-}
 
 template <int BMODE, int NT1>
 __global__ void __launch_bounds__(2 * NT1, NT1 == NT_NARROW ? 3 : 2)
@@ -698,10 +674,14 @@ __global__ void __launch_bounds__(2 * NT1, NT1 == NT_NARROW ? 3 : 2)
   const int c = b0 - HL1 + t;
   if (forward) {
     PlusForward<BMODE, NT1> sw(R, a, k, t, c, a0, a1);
-    run_role(sw, &R.A[0][sw.u], s_begin, s_end, s_lo, s_hi);
+    float* ringA = &R.A[0][sw.u];
+#pragma unroll 1
+    for (int s = s_begin - (AHEAD + 1); s < s_begin; ++s)
+      sw.template request<false>(s, RowsRT<RingsPlus<NT1>::W>{ringA, s});
+    sweep_band(sw, ringA, s_begin, s_end, s_lo, s_hi);
   } else {
     PlusBackward<BMODE, NT1> sw(R, a, k, t, c, b0, b1, a0, a1);
-    run_role(sw, &R.A[0][sw.u], s_begin, s_end, s_lo, s_hi);
+    sweep_band(sw, &R.A[0][sw.u], s_begin, s_end, s_lo, s_hi);
   }
 }
 
@@ -757,8 +737,8 @@ struct CrossSweep {
     xin = a.x + plane * a.x_sc + (int64_t)clampi(c, 0, m - 1) * a.x_sw +
           (int64_t)clampi(a0 - 5 - (AHEAD + 1) + 2, 0, n - 1) * x_sh;
     cg = c >= -BWD_GHOST && c < m + BWD_GHOST;
-    ws_ld = a.m + 2 * BWD_GHOST;
-    const int64_t cells = (a.n + 2 * BWD_GHOST) * ws_ld;
+    ws_ld = a.ws_ld;
+    const int64_t cells = a.ws_cells;
     ws_ab = cells - 3 * ws_ld;
     const int s0 = a0 - 5;  // first step (requests start AHEAD + 1 steps before it)
     wxb = a.ws + plane * 2 * cells + (int64_t)(s0 - (AHEAD + 1) - 1 + BWD_GHOST) * ws_ld + (c + BWD_GHOST);
@@ -956,7 +936,8 @@ struct SweepModel {
 // resident), the others short bands on an idle GPU; latencies of 0.5 to 0.75
 // and 0.3 to 0.5 us and fills 25% off choose shapes within 2% of each other.
 // Bands of at least 16 rows, the rule before, left small images on a few CTAs:
-// 3x64x64 39.5 -> 23.0 us, 1x128x200 -> 23.6, 3x256x256 43.3 -> 40.5.
+// 3x64x64 39.5 -> 23.0 us, 3x256x256 43.3 -> 40.5 (then 20.8 and 35.9 with the
+// requests moved).
 constexpr SweepModel PLUS_MODEL = {0.50f, {0.31f, 0.46f}, 13.f};
 constexpr SweepModel CROSS_MODEL = {0.30f, {0.133f, 0.20f}, 10.f};
 
@@ -1053,8 +1034,11 @@ size_t bwd_workspace_bytes(int64_t n, int64_t m, int64_t planes) {
          (size_t)planes;
 }
 
-cudaError_t launch_zoom2x_bwd(const BwdArgs& a, const MethodConsts& k, int bmode,
+cudaError_t launch_zoom2x_bwd(const BwdArgs& args, const MethodConsts& k, int bmode,
                               cudaStream_t stream) {
+  BwdArgs a = args;
+  a.ws_ld = a.m + 2 * BWD_GHOST;
+  a.ws_cells = (a.n + 2 * BWD_GHOST) * a.ws_ld;
   switch (bmode) {
     case B2: return launch_all<B2>(a, k, stream);
     case B0: return launch_all<B0>(a, k, stream);

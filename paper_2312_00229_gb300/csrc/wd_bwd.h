@@ -21,6 +21,7 @@ struct BwdArgs {
   int64_t gi_sc, gi_sh, gi_sw;
   int64_t orows, ocols;
   int g_vec;  // output-gradient columns 2c, 2c + 1 load as one aligned float2
+  int64_t ws_ld, ws_cells;  // workspace row stride and plane size (set by the launcher)
   float* ws;  // 2 * (n + 2 BWD_GHOST) * (m + 2 BWD_GHOST) * planes floats
 };
 
