@@ -19,7 +19,7 @@ struct FwdArgs {
   int64_t rows_per_band;
   int out_vec;                   // unit column stride and 2-element aligned rows
   int out_vec4;                  // unit column stride and 4-element aligned rows
-  int threads;                   // CTA width: 256 or 128 (one column), 128 or 64 (two)
+  int threads;                   // CTA width: 256 or 128 (one column), 128, 96 or 64 (two)
   int cols;                      // coarse columns per thread: 1, or 2 (paired tile)
 };
 
@@ -34,7 +34,7 @@ __host__ __device__ inline void set_store_modes(FwdArgs& a, int64_t esz) {
 
 // Tile shape of a one-launch forward: `threads` per CTA, `cols` coarse columns
 // per thread (1: 256 or 128 threads, 247 or 119 output columns per strip; 2:
-// 128 or 64 threads, 246 or 118) and coarse rows per band.
+// 128, 96 or 64 threads, 246, 182 or 118) and coarse rows per band.
 struct FwdPlan {
   int threads, cols;
   int64_t rows;

@@ -42,12 +42,14 @@ __global__ void __launch_bounds__(NT, 3 * 128 / NT)
 template <int BMODE, class IO>
 cudaError_t launch_fwd(const FwdArgs& a, const MethodConsts& k, cudaStream_t stream) {
   if (a.cols == 2) {
-    const int nt = a.threads == 64 ? 64 : 128;
+    const int nt = a.threads == 64 || a.threads == 96 ? a.threads : 128;
     const int64_t tw = 2 * nt - 10;
     dim3 grid((unsigned)((a.m + tw - 1) / tw),
               (unsigned)((a.n + a.rows_per_band - 1) / a.rows_per_band), (unsigned)a.planes);
     if (nt == 64)
       zoom2x_fwd_kernel2<BMODE, IO, 64><<<grid, nt, 0, stream>>>(a, k);
+    else if (nt == 96)
+      zoom2x_fwd_kernel2<BMODE, IO, 96><<<grid, nt, 0, stream>>>(a, k);
     else
       zoom2x_fwd_kernel2<BMODE, IO, 128><<<grid, nt, 0, stream>>>(a, k);
     return cudaGetLastError();

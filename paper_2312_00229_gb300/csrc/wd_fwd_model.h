@@ -11,7 +11,7 @@
 // the sweep is a serial chain: 3x48x64 uint8 14.0 -> 6.2 us (rows 16 -> 3),
 // 3x256x256 FP32 15.2 -> 9.2 us, 1x300x700 FP16 14.4 -> 8.3 us, 3x512x512
 // 17.9 -> 15.9 us; from 1024x1024 on the plans are those of the rule before
-// (two-column strips, bands balancing the waves).
+// (two-column strips, bands balancing the waves), or 182-column strips.
 #pragma once
 
 #include <stdint.h>
@@ -27,9 +27,13 @@ struct FwdShape {
 constexpr float FWD_FILL = 6.3f;    // steps
 constexpr float FWD_LAUNCH = 2.2f;  // us
 
-// index 0 .. 3: strips of 118, 246, 119, 247 output columns
-constexpr FwdShape FWD_SHAPES[4] = {{64, 2, 6, 0.5365f, 0.1250f},
+// Strips of 118, 246, 182, 119 and 247 output columns.  (182 is the library's
+// own choice only: it covers 512 columns with 576 thread columns where 118 takes
+// 640 and 246 takes 768, 96x512x512 FP32 279 -> 247 us, 3x512x512 uint8 15.9 -> 14.3,
+// 3x480x854 18.7 -> 17.9; on a tie 118 is kept, 1-2% faster.)
+constexpr FwdShape FWD_SHAPES[5] = {{64, 2, 6, 0.5365f, 0.1250f},
                                     {128, 2, 3, 0.4970f, 0.2580f},
+                                    {96, 2, 4, 0.5365f, 0.1915f},
                                     {128, 1, 4, 0.3846f, 0.1481f},
                                     {256, 1, 2, 0.3840f, 0.3031f}};
 

@@ -18,7 +18,8 @@ def _img(shape, seed, dtype=torch.uint8):
 
 @pytest.mark.parametrize("c,n,m", [(1, 1, 1), (3, 2, 7), (1, 3, 400), (3, 17, 118), (3, 48, 64),
                                    (1, 119, 119), (2, 200, 247), (3, 333, 500), (1, 1024, 130),
-                                   (65, 40, 246), (3, 700, 900)])
+                                   (65, 40, 246), (3, 700, 900), (3, 512, 512), (1, 30, 182),
+                                   (8, 64, 364), (24, 100, 183), (3, 300, 545)])
 @pytest.mark.parametrize("mode", [0, 1])
 def test_default_plan_bits(c, n, m, mode):
     x = _img((c, n, m), 7 * n + m)
