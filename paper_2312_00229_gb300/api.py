@@ -147,8 +147,8 @@ def zoom2x_fwd(x: torch.Tensor, params: Optional[Params] = None, out_dtype=None,
 
     ``rows_per_tile``: band height per CTA; None = the autotuner's cached
     choice for this size class (see ``autotune``), 0 = the library default.
-    ``tile_width``: output columns per CTA, 247 (256 threads) or 119 (128
-    threads); 0 = the library's choice for the image width."""
+    ``tile_width``: output columns per CTA, 247, 119, 246 or 118 (see
+    ``autotune``); 0 = the library's choice."""
     params = params or _DEFAULT
     _require_cuda(x, "x")
     if x.numel() == 0:

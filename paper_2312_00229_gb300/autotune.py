@@ -5,15 +5,15 @@ parameter, and the strip width (output columns per CTA) as one of the built
 tile shapes, which also fix the coarse columns per thread (the threads that
 share one quad column's work): 247 (256 threads, one column each), 119 (128
 threads, one column), 246 (128 threads, two columns each) or 118 (64
-threads, two columns).  The one-launch forward picks a shape from the image
-width; the batched launch takes one of the one-column widths from the
-caller.  This module times candidate shapes
+threads, two columns).  Left to itself the library picks the shape of least
+modelled time for the image's size (one launch) or for all of a batch's.
+This module times candidate shapes
 on the current GPU with CUDA events and caches the fastest per size class in
 a JSON file, keyed by device name, storage types, layout and size class
 (planes and the image sides rounded up to powers of two).
 
 ``api.zoom2x_fwd(..., rows_per_tile=None)`` consults the cache; a miss uses the
-library's own default (the band count that balances the last wave of CTAs).
+library's own default.
 """
 from __future__ import annotations
 

@@ -960,7 +960,7 @@ SweepShape pick_shape(const SweepModel& model, const int (&occ)[2], const int (&
     };
     const double full = step(occ[i]);
     int64_t last = -1;
-    for (int64_t b = 1; b <= rows_total && b <= 65535; ++b) {
+    for (int64_t b = 1; b <= rows_total && b <= 4096; ++b) {
       const int64_t rows = (rows_total + b - 1) / b;
       if (rows == last) continue;
       // bands below 16 rows only where they still find idle CTA slots

@@ -52,7 +52,7 @@ FwdPlan find_plan(const PlanKey& q) {
     const int64_t slots = (int64_t)q.sms * s.per_sm;
     const double full = step_us(s, s.per_sm);
     int64_t last = -1;
-    for (int64_t bands = 1; bands <= q.n; ++bands) {
+    for (int64_t bands = 1; bands <= q.n && bands <= 4096; ++bands) {
       const int64_t rows = q.rows > 0 ? q.rows : (q.n + bands - 1) / bands;
       if (rows == last) continue;
       // bands below 16 rows only where they still find idle CTA slots
