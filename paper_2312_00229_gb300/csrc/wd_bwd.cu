@@ -679,6 +679,7 @@ __global__ void __launch_bounds__(2 * NT1, NT1 == NT_NARROW ? 3 : 2)
     for (int s = s_begin - (AHEAD + 1); s < s_begin; ++s)
       sw.template request<false>(s, RowsRT<RingsPlus<NT1>::W>{ringA, s});
     sweep_band(sw, ringA, s_begin, s_end, s_lo, s_hi);
+    copy_wait<0>();  // no copy lands in shared memory after the CTA
   } else {
     PlusBackward<BMODE, NT1> sw(R, a, k, t, c, b0, b1, a0, a1);
     sweep_band(sw, &R.A[0][sw.u], s_begin, s_end, s_lo, s_hi);
@@ -906,6 +907,7 @@ __global__ void __launch_bounds__(NT2, NT2 == NT_NARROW ? 4 : 2)
   const int s_lo = max(sw.a0, 0) + 8;
   const int s_hi = min(sw.a1 + 5, sw.n + 2);
   sweep_band(sw, &R.A[0][sw.u], s_begin, s_end, s_lo, s_hi);
+  copy_wait<0>();  // no copy lands in shared memory after the CTA
 }
 
 // Resident CTAs per SM of a kernel with `smem` bytes of dynamic shared memory,
