@@ -284,14 +284,17 @@ __device__ __forceinline__ void rs_flush(char* out, int64_t sw, int vec4,
 // columns, four per lane.  Either way the encoded outputs go through a staging
 // row in shared memory to whole-word stores.
 //
-// What bounds it: instruction issue (70% of slots at 3x uint8; FMA pipe 47%, LSU
-// 44%), a third of it address arithmetic.  Against the form before (a decoded
+// What bounds it: instruction issue (71% of slots at 3x uint8; FMA pipe 46%, LSU
+// 44%), a quarter of it address arithmetic.  Against the form before (a decoded
 // window in shared memory, every output's indicators formed anew, 4-byte
 // stores from four outputs per lane with strided z reads), us:
-//     1080p uint8 -> 3x 124 -> 79, -> 2x 77 -> 48, -> 1.33x 39.9 -> 33.5, 1x 33 -> 26
-//     4317x7677 FP32 -> 3240x5760 uint8 353 -> 224; 1080p FP32 -> 900x1600 26 -> 20
+//     1080p uint8 -> 3x 124 -> 75, -> 2x 77 -> 45, -> 1.33x 39.9 -> 31.6, 1x 33 -> 24.5
+//     4317x7677 FP32 -> 3240x5760 uint8 353 -> 214; 1080p FP32 -> 900x1600 26 -> 19.4
+// (79, 48, 33.5, 26, 224 and 20 before windows inside the image took their rows one
+// stride apart without the clamped offsets, and the rows of each cell were
+// counted once per warp).
 // Small outputs are bound by the launch and one warp's chain: 200x300 -> 500x700
-// 5.0 -> 5.3, 64x64 -> 8x 4.7 -> 6.2 (nine outputs a cell, in turn), 100x100 from
+// 5.0 -> 5.2, 64x64 -> 8x 4.7 -> 6.1 (nine outputs a cell, in turn), 100x100 from
 // 64x64 4.7 -> 3.3.  Packed constants pinned in registers, scalar instead of
 // packed arithmetic, and two or four CTAs per SM measured slower.
 template <bool UP>
@@ -310,28 +313,44 @@ struct RsShared {
   __align__(16) unsigned char stage[RS_WARPS][4 * (UP ? RS_TC_MAX : RS_TC_DOWN) + 16];
 };
 
-// Pass 1 of a warp: z of its `nq` output rows (tile rows q0 ..) at window
-// columns k0 + lane and k0 + lane + 32 (columns past the window repeat the
-// last and are not used).  in_base: input row of in_off[0].
+// Pass 1 of a warp: z of its output rows (tile rows q0 ..) at window columns
+// k0 + lane and k0 + lane + 32 (those past the window are not used).  rows_in:
+// input rows they read; rows_of: output rows in each cell, four bits a cell;
+// in_base: input row of in_off[0].
 template <int BMODE, class TIn, class SH>
 __device__ __forceinline__ void column_pass(const ResampleArgs& a, SH& sh, int warp, int lane,
-                                            int q0, int nq, int in_base, int kfirst, int wc,
+                                            int q0, int rows_in, uint32_t rows_of, int in_base,
+                                            int kfirst, int wc,
                                             int k0, const char* plane, int esz, float eps,
                                             float beta) {
   const int ka = k0 + lane, kb = ka + 32;
-  const char* pa = plane + (int64_t)clamp_idx(kfirst + min(ka, wc - 1), (int)a.m) * a.in_sw * esz;
-  const char* pb = plane + (int64_t)clamp_idx(kfirst + min(kb, wc - 1), (int)a.m) * a.in_sw * esz;
-  // lane q holds the cell of row q, counted from the first row's
   const int first = sh.row_i[q0];
-  const int rel = lane < nq ? sh.row_i[q0 + lane] - first : -1;
-  const int rows_in = __shfl_sync(0xffffffffu, rel, nq - 1) + 4;  // input rows they read
-  const int64_t* off = sh.in_off + (first - 1 - in_base);
   uint32_t ba[RS_PRE], bb[RS_PRE];
+  if (a.in_sw == 1 && kfirst >= 0 && kfirst + k0 + 64 <= (int)a.m && first >= 1 &&
+      first - 1 + rows_in <= (int)a.n) {
+    // (uniform) nothing to clamp: rows one stride apart, columns at fixed offsets
+    const char* p0 = plane + (int64_t)(first - 1) * a.in_sh * esz + (kfirst + ka) * esz;
+    const int64_t step = a.in_sh * esz;
 #pragma unroll
-  for (int p = 0; p < RS_PRE; ++p) {
-    if (p < rows_in) {  // (uniform)
-      ba[p] = rs_load_bits<TIn>(pa + off[p], 0, a.in_dtype);
-      bb[p] = rs_load_bits<TIn>(pb + off[p], 0, a.in_dtype);
+    for (int p = 0; p < RS_PRE; ++p) {
+      if (p < rows_in) {
+        ba[p] = rs_load_bits<TIn>(p0, 0, a.in_dtype);
+        bb[p] = rs_load_bits<TIn>(p0, 32, a.in_dtype);
+        p0 += step;
+      }
+    }
+  } else {
+    const char* pa =
+        plane + (int64_t)clamp_idx(kfirst + min(ka, wc - 1), (int)a.m) * a.in_sw * esz;
+    const char* pb =
+        plane + (int64_t)clamp_idx(kfirst + min(kb, wc - 1), (int)a.m) * a.in_sw * esz;
+    const int64_t* off = sh.in_off + (first - 1 - in_base);
+#pragma unroll
+    for (int p = 0; p < RS_PRE; ++p) {
+      if (p < rows_in) {  // (uniform)
+        ba[p] = rs_load_bits<TIn>(pa + off[p], 0, a.in_dtype);
+        bb[p] = rs_load_bits<TIn>(pb + off[p], 0, a.in_dtype);
+      }
     }
   }
   f2 v[RS_PRE];
@@ -345,7 +364,7 @@ __device__ __forceinline__ void column_pass(const ResampleArgs& a, SH& sh, int w
   const float2* rh = sh.row_h + q0;
 #pragma unroll
   for (int p = 0; p < RS_CELLS; ++p) {
-    int rows = __popc(__ballot_sync(0xffffffffu, rel == p));  // output rows in cell p
+    int rows = (rows_of >> (4 * p)) & 15;  // output rows in cell p
     if (rows) {
       const Cell2 c = cell2<BMODE>(v[p], v[p + 1], v[p + 2], v[p + 3], eps, beta);
 #pragma unroll 1
@@ -492,8 +511,13 @@ __global__ void __launch_bounds__(RS_THREADS, 3)
   const int nq = min(nr - q0, a.warp_rows);
   if (nq <= 0) return;
   const char* in_plane = static_cast<const char*>(a.in) + plane * a.in_sc * esz;
+  // lane q holds the cell of row q, counted from the first row's
+  const int rel = lane < nq ? sh.row_i[q0 + lane] - sh.row_i[q0] : -1;
+  const int rows_in = __shfl_sync(0xffffffffu, rel, nq - 1) + 4;
+  uint32_t rows_of = rel >= 0 ? 1u << (4 * rel) : 0u;
+  rows_of = __reduce_add_sync(0xffffffffu, rows_of);
   for (int k0 = 0; k0 < wc; k0 += 64)
-    column_pass<BMODE, TIn>(a, sh, warp, lane, q0, nq, in_base, kfirst, wc, k0, in_plane, esz, eps,
+    column_pass<BMODE, TIn>(a, sh, warp, lane, q0, rows_in, rows_of, in_base, kfirst, wc, k0, in_plane, esz, eps,
                             beta);
   __syncwarp();
   const int osz = elem_bytes<TOut>(a.out_dtype);
