@@ -160,7 +160,7 @@ def zoom2x_fwd(x: torch.Tensor, params: Optional[Params] = None, out_dtype=None,
         rows_per_tile, width = autotune.lookup_shape(x, out.dtype, layout)
         tile_width = tile_width or width
     rc = B.weno_zoom2x_fwd_tiled(image(x, layout), _DT[x.dtype], image(out, layout),
-                                 _DT[out.dtype], _params_c(params), rows_per_tile, tile_width,
+                                 _DT[out.dtype], _params_c(params), rows_per_tile, int(tile_width),
                                  _stream(x.device))
     B.check("weno_zoom2x_fwd", rc)
     return out
