@@ -23,6 +23,7 @@
 #include "wd_common.cuh"
 #include "wd_packed.cuh"
 #include "wd_resample.h"
+#include "wd_resample_window.h"
 
 namespace wdweno {
 
@@ -326,10 +327,10 @@ __device__ __forceinline__ void column_pass(const ResampleArgs& a, SH& sh, int w
   const int ka = k0 + lane, kb = ka + 32;
   const int first = sh.row_i[q0];
   uint32_t ba[RS_PRE], bb[RS_PRE];
-  if (a.in_sw == 1 && kfirst >= 0 && kfirst + k0 + 64 <= (int)a.m && first >= 1 &&
-      first - 1 + rows_in <= (int)a.n) {
+  if (a.in_sw == 1 && window_inside(kfirst, k0, (int)a.m, first, rows_in, (int)a.n)) {
     // (uniform) nothing to clamp: rows one stride apart, columns at fixed offsets
-    const char* p0 = plane + (int64_t)(first - 1) * a.in_sh * esz + (kfirst + ka) * esz;
+    const char* p0 =
+        plane + (int64_t)(first - 1) * a.in_sh * esz + column_bytes(kfirst, ka, esz);
     const int64_t step = a.in_sh * esz;
 #pragma unroll
     for (int p = 0; p < RS_PRE; ++p) {
