@@ -127,7 +127,11 @@ def _level_out(x: torch.Tensor, params: Params, layout: str, dtype) -> torch.Ten
     with planar rows padded to a multiple of four elements.  Only the next
     level reads it, and rows that all start on a four-element boundary are
     written with one vector store per thread and fine row (odd widths of the
-    2n-1 grid otherwise take three)."""
+    2n-1 grid otherwise take three).  What the zoom refuses is refused before
+    the allocation."""
+    _require_cuda(x, "x")
+    if x.numel() == 0:
+        raise ValueError("empty input")
     h, w = out_hw(x.shape[-2], x.shape[-1], params)
     if layout == "hwc" or w % 4 == 0:
         return _out_like(x, params, layout, dtype)
