@@ -119,7 +119,7 @@ def tune_fwd(x: torch.Tensor, params=None, out_dtype=None, layout: str = "chw",
              candidates: Iterable[int] = CANDIDATES, widths: Iterable[int] = (0,) + TILE_WIDTHS,
              reps: int = 10) -> Dict[Tuple[int, int], float]:
     """Times each candidate (band height, tile width) on `x` and caches the
-    fastest (width 0 = the library's choice for the image width).
+    fastest (width 0 = the library's choice).
     Returns {(rows_per_tile, tile_width): milliseconds}."""
     from . import api
     params = params or api.Params()
@@ -170,18 +170,29 @@ def tune_cascade(x: torch.Tensor, levels: int, params=None, out_dtype=None,
 
 
 def _batched_key(images: Sequence[torch.Tensor], out_dtype, layout: str) -> str:
-    return "|".join(["batched", _device_name(images[0].device),
-                     str(images[0].dtype), str(out_dtype or images[0].dtype), layout,
-                     str(_pow2(len(images)))])
+    """Size class of a batch: storage types, layout, and, rounded up to powers
+    of two, the image count, the largest sides and the mean of the samples per
+    image.  (Under the count alone, the height of 128 rows that suits five
+    large images was also taken for five small ones, where it leaves most of
+    the GPU idle.)"""
+    from .api import _planes
+    head = ["batched", _device_name(images[0].device), str(images[0].dtype),
+            str(out_dtype or images[0].dtype), layout, str(_pow2(len(images)))]
+    sides = [tuple(map(int, _planes(im, layout)[:3])) for im in images]
+    mean = sum(h * w * c for h, w, c in sides) // len(sides)
+    return "|".join(head + [str(_pow2(max(h for h, _, _ in sides))),
+                            str(_pow2(max(w for _, w, _ in sides))), str(_pow2(mean))])
 
 
 def tune_batched(images: Sequence[torch.Tensor], params=None, out_dtype=None,
-                 layout: str = "chw", candidates: Iterable[int] = (16, 32, 64, 128),
+                 layout: str = "chw", candidates: Iterable[int] = (0, 16, 32, 64, 128),
                  widths: Iterable[int] = BATCHED_TILE_WIDTHS,
                  reps: int = 5) -> Dict[Tuple[int, int], float]:
     """Times the persistent batched launch for each (band height, tile width)
-    and caches the fastest under the batch's size class (dtype, layout, image
-    count).  Returns {(rows_per_tile, tile_width): milliseconds}."""
+    and caches the fastest under the batch's size class (see
+    ``_batched_key``).  Height 0 is the one chosen on the device from the
+    images' sizes: where it is the fastest, that choice is what is kept.
+    Returns {(rows_per_tile, tile_width): milliseconds}."""
     from . import api
     times = {}
     for tw in widths:
@@ -201,6 +212,9 @@ def lookup_batched(images: Sequence[torch.Tensor], out_dtype,
                    layout: str) -> Tuple[int, int]:
     """Cached (band height, tile width) of this batch's size class, or (0, 0)
     (the library defaults)."""
-    key = _batched_key(images, out_dtype, layout)
+    images[0]  # (an empty sequence is an error with and without a cache)
     cache = _load()
+    if not cache:
+        return 0, 0
+    key = _batched_key(images, out_dtype, layout)
     return cache.get(key, 0), cache.get(key + "|tile_width", 0)
