@@ -132,6 +132,7 @@ def _level_out(x: torch.Tensor, params: Params, layout: str, dtype) -> torch.Ten
     _require_cuda(x, "x")
     if x.numel() == 0:
         raise ValueError("empty input")
+    dtype = dtype or x.dtype  # (as the zoom's own output: None keeps the input's)
     h, w = out_hw(x.shape[-2], x.shape[-1], params)
     if layout == "hwc" or w % 4 == 0:
         return _out_like(x, params, layout, dtype)
