@@ -16,13 +16,13 @@
 // Everything of an interpolant but C_s and the powers of t belongs to its
 // cell, not to t: g, sL, sR and the weights' powers of the indicators are
 // formed once per cell (Cell2) and evaluated at each output inside (eval2).
-#include <algorithm>
 #include <atomic>
 #include <type_traits>
 
 #include "wd_common.cuh"
 #include "wd_packed.cuh"
 #include "wd_resample.h"
+#include "wd_resample_plan.h"
 #include "wd_resample_window.h"
 
 namespace wdweno {
@@ -151,31 +151,15 @@ __device__ __forceinline__ void rs_store(void* base, int64_t idx, float v, int d
   }
 }
 
-template <class T>
-__device__ __forceinline__ void rs_store4(void* base, int64_t idx, const float (&u)[4], int dt,
-                                          int clampf) {
-  if constexpr (std::is_same<T, Dyn>::value) {
-    store4_vec(base, idx, u[0], u[1], u[2], u[3], dt, clampf);
-  } else {
-    store4_typed<T>(base, idx, u[0], u[1], u[2], u[3], clampf);
-  }
-}
-
 // One thread per output, for reductions beyond 1/2 (little to share between
-// neighbouring outputs) and single-sample axes: all 16 loads are issued before
-// the first is used, columns are interpolated in packed pairs.  1080p ->
-// 480x270 uint8: 9.2 us with run-time types and 64-bit positions, now 6.8.
-template <int BMODE, class TIn, class TOut>
-__global__ void __launch_bounds__(256) resample_kernel(ResampleArgs a, float eps, float beta) {
-  const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t r = (int64_t)blockIdx.y * blockDim.y + threadIdx.y;
-  if (r >= a.n_out || c >= a.m_out) return;
-  const int64_t plane = blockIdx.z;
+// neighbouring outputs) and single-sample axes: all 16 loads are issued before the first is used,
+// columns are interpolated in packed pairs.  1080p -> 480x270 uint8: 9.2 us with
+// run-time types and 64-bit positions, now 6.8.
+//
+template <int BMODE, class TIn>
+__device__ __forceinline__ float output_at(const ResampleArgs& a, int64_t plane, int i, float ty,
+                                           int j, float tx, float eps, float beta) {
   const int n = (int)a.n, m = (int)a.m;
-  int i, j;
-  float ty, tx;
-  grid_pos((int)r, n, (int)a.n_out, a.div_y, i, ty);
-  grid_pos((int)c, m, (int)a.m_out, a.div_x, j, tx);
   int64_t row[4], col[4];
 #pragma unroll
   for (int p = 0; p < 4; ++p) {
@@ -205,23 +189,28 @@ __global__ void __launch_bounds__(256) resample_kernel(ResampleArgs a, float eps
                                   beta),
                      pk_bc(tx), pk_bc(pos_c0(tx)), pk_bc(pos_h(tx)))
             .x;
+  return u;
+}
+
+template <int BMODE, class TIn, class TOut>
+__global__ void __launch_bounds__(256) resample_kernel(ResampleArgs a, float eps, float beta) {
+  const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t r = (int64_t)blockIdx.y * blockDim.y + threadIdx.y;
+  if (r >= a.n_out || c >= a.m_out) return;
+  const int64_t plane = blockIdx.z;
+  const int n = (int)a.n, m = (int)a.m;
+  int i, j;
+  float ty, tx;
+  grid_pos((int)r, n, (int)a.n_out, a.div_y, i, ty);
+  grid_pos((int)c, m, (int)a.m_out, a.div_x, j, tx);
+  const float u = output_at<BMODE, TIn>(a, plane, i, ty, j, tx, eps, beta);
   rs_store<TOut>(a.out, plane * a.out_sc + r * a.out_sh + c * a.out_sw, u, a.out_dtype,
                  a.clamp_float);
 }
 
-// Tile sizes of the tiled form below.
-constexpr int RS_WARPS = 8;
+// ---- the tiled forms (sizes: wd_resample_plan.h) -------------------------------------
 constexpr int RS_THREADS = 32 * RS_WARPS;
-constexpr int RS_MAX_ROWS = 8;                 // output rows per warp, at most
-constexpr int RS_DOWN_ROWS = 4;                // the same, where the rows are reduced
-constexpr int RS_CELLS = 8;                    // input cells a warp's rows span, at most
-constexpr int RS_PRE = RS_CELLS + 3;           // input rows
-constexpr int RS_TC_DOWN = 128;                // output columns of a tile, reduced
-constexpr int RS_TC_MAX = 480;                 // and at most, magnified
-constexpr int RS_WC_UP = 64;                   // window columns, magnified
-constexpr int RS_WC_DOWN = 2 * RS_TC_DOWN + 8; // (>= 2 (RS_TC_DOWN - 1) + 5)
-constexpr int RS_MAX_IN = 2 * RS_WARPS * RS_DOWN_ROWS + 8;  // input rows of a tile, at most
-constexpr int RS_REG_OUT = 4;                  // outputs of a cell with constants in registers
+constexpr int RS_REG_OUT = 4;  // outputs of a cell with constants in registers
 
 template <class T>
 __device__ __forceinline__ int elem_bytes(int dt) {
@@ -279,11 +268,17 @@ __device__ __forceinline__ void rs_flush(char* out, int64_t sw, int vec4,
 // Per output this is 1 + (in/out column ratio) + halo 1-D interpolants
 // instead of the 5 of the direct form.
 //
-// Magnified columns (UP): the tile is as wide as fits 64 window columns, two
-// per lane, and pass 2 gives a lane two cells of the row, whose indicators
-// serve all of their outputs (three at 3x).  Reduced columns: 128 output
-// columns, four per lane.  Either way the encoded outputs go through a staging
-// row in shared memory to whole-word stores.
+// The forms differ in the tile and in pass 2 (which one runs: wd_resample_plan.h):
+//   RS_CELLS    magnified columns: the tile is as wide as fits 64 window columns,
+//               two per lane, and pass 2 gives a lane two cells of the row,
+//               whose indicators serve all of their outputs (three at 3x)
+//   RS_OUTPUTS  the outputs of 128 window columns, 128 at most, and up to eight
+//               rows a warp; pass 2 gives a lane up to four outputs, each with
+//               its cell's indicators formed anew
+//   RS_REDUCED  128 outputs, four rows a warp, up to 264 window columns; pass 2
+//               by outputs
+// The encoded outputs go through a staging row in shared memory to whole-word
+// stores.
 //
 // What bounds it: instruction issue (71% of slots at 3x uint8; FMA pipe 46%, LSU
 // 44%), a quarter of it address arithmetic.  Against the form before (a decoded
@@ -294,24 +289,25 @@ __device__ __forceinline__ void rs_flush(char* out, int64_t sw, int vec4,
 // (79, 48, 33.5, 26, 224 and 20 before windows inside the image took their rows one
 // stride apart without the clamped offsets, and the rows of each cell were
 // counted once per warp).
-// Small outputs are bound by the launch and one warp's chain: 200x300 -> 500x700
-// 5.0 -> 5.2, 64x64 -> 8x 4.7 -> 6.1 (nine outputs a cell, in turn), 100x100 from
-// 64x64 4.7 -> 3.3.  Packed constants pinned in registers, scalar instead of
-// packed arithmetic, and two or four CTAs per SM measured slower.
-template <bool UP>
+// Small outputs are bound by the launch and one warp's chain: 64x64 -> 100x100 4.7
+// -> 3.3 us.  Packed constants pinned in registers, scalar instead of packed
+// arithmetic, and two or four CTAs per SM measured slower.
+template <int FORM>
 struct RsShared {
-  static constexpr int TC = UP ? RS_TC_MAX : RS_TC_DOWN;
-  static constexpr int WZ = UP ? RS_WC_UP + 4 : RS_WC_DOWN;
+  static constexpr int TC = FORM == RS_CELLS ? RS_TC_MAX : RS_TC_DOWN;
+  static constexpr int WZ =
+      FORM == RS_CELLS ? RS_WC_UP + 4 : (FORM == RS_OUTPUTS ? RS_WC_OUT : RS_WC_DOWN);
+  static constexpr int ROWS = FORM == RS_REDUCED ? RS_DOWN_ROWS : RS_MAX_ROWS;  // a warp, at most
   float4 row_a[RS_WARPS * RS_MAX_ROWS];  // (t, t, C0, C0) of each output row
   float2 row_h[RS_WARPS * RS_MAX_ROWS];  // (h, h)
   int64_t in_off[RS_MAX_IN];             // byte offset of each (clamped) input row
   int row_i[RS_WARPS * RS_MAX_ROWS];     // its cell
   int col_j[TC];
   float col_t[TC];
-  int start[RS_WC_UP + 1];               // first output column of each cell (UP)
-  float z[RS_WARPS][UP ? RS_MAX_ROWS : RS_DOWN_ROWS][WZ];
+  int start[RS_WC_UP + 1];               // first output column of each cell (RS_CELLS)
+  float z[RS_WARPS][ROWS][WZ];
   // encoded outputs of a row, and a spare element
-  __align__(16) unsigned char stage[RS_WARPS][4 * (UP ? RS_TC_MAX : RS_TC_DOWN) + 16];
+  __align__(16) unsigned char stage[RS_WARPS][4 * TC + 16];
 };
 
 // Pass 1 of a warp: z of its output rows (tile rows q0 ..) at window columns
@@ -364,7 +360,7 @@ __device__ __forceinline__ void column_pass(const ResampleArgs& a, SH& sh, int w
   const float4* ra = sh.row_a + q0;
   const float2* rh = sh.row_h + q0;
 #pragma unroll
-  for (int p = 0; p < RS_CELLS; ++p) {
+  for (int p = 0; p < RS_MAX_CELLS; ++p) {
     int rows = (rows_of >> (4 * p)) & 15;  // output rows in cell p
     if (rows) {
       const Cell2 c = cell2<BMODE>(v[p], v[p + 1], v[p + 2], v[p + 3], eps, beta);
@@ -381,7 +377,7 @@ __device__ __forceinline__ void column_pass(const ResampleArgs& a, SH& sh, int w
   }
 }
 
-// Pass 2 of a warp on magnified columns: cells of at most NJ outputs, whose
+// Pass 2 of a warp by cells: of at most NJ outputs, whose
 // positions are kept in registers (with NJ = RS_REG_OUT cells may have more,
 // which read theirs from the tables).
 template <int BMODE, class TOut, int NJ, class SH>
@@ -433,12 +429,13 @@ __device__ __forceinline__ void row_pass_up(const ResampleArgs& a, SH& sh, int w
   }
 }
 
-// Pass 2 of a warp on reduced columns: outputs lane, lane + 32, .. of the row
-// (consecutive lanes read z values 1 to 2 apart), two in a packed pair.
+// Pass 2 of a warp by outputs: outputs lane, lane + 32, .. of the row
+// (consecutive lanes read z values at most 2 apart), two in a packed pair.
 template <int BMODE, class TOut, class SH>
-__device__ __forceinline__ void row_pass_down(const ResampleArgs& a, SH& sh, int warp, int lane,
+__device__ __forceinline__ void row_pass_outputs(const ResampleArgs& a, SH& sh, int warp, int lane,
                                               int nq, int nc, int kfirst, char* out,
                                               int64_t row_bytes, float eps, float beta) {
+  constexpr bool FORM_OUT = SH::ROWS != RS_DOWN_ROWS;
   const float* z[4];
   f2 t[2], C0[2], h[2];
 #pragma unroll
@@ -452,10 +449,11 @@ __device__ __forceinline__ void row_pass_down(const ResampleArgs& a, SH& sh, int
   }
   unsigned char* stage = sh.stage[warp];
 #pragma unroll
-  for (int r = 0; r < RS_DOWN_ROWS; ++r, out += row_bytes) {
+  for (int r = 0; r < SH::ROWS; ++r, out += row_bytes) {
     if (r >= nq) break;
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
+      if (FORM_OUT && q == 1 && nc <= 64) break;  // (uniform)
       const float* za = z[2 * q] + r * SH::WZ;
       const float* zb = z[2 * q + 1] + r * SH::WZ;
       const f2 u = eval2<BMODE>(
@@ -472,10 +470,10 @@ __device__ __forceinline__ void row_pass_down(const ResampleArgs& a, SH& sh, int
   }
 }
 
-template <int BMODE, class TIn, class TOut, bool UP>
+template <int BMODE, class TIn, class TOut, int FORM>
 __global__ void __launch_bounds__(RS_THREADS, 3)
     resample_tiled_kernel(const __grid_constant__ ResampleArgs a, float eps, float beta) {
-  using SH = RsShared<UP>;
+  using SH = RsShared<FORM>;
   __shared__ SH sh;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int n = (int)a.n, m = (int)a.m;
@@ -497,12 +495,12 @@ __global__ void __launch_bounds__(RS_THREADS, 3)
   }
   __syncthreads();
   const int kfirst = sh.col_j[0] - 1, in_base = sh.row_i[0] - 1;
-  const int wc = sh.col_j[nc - 1] + 2 - kfirst + 1;  // <= RS_WC_UP, RS_WC_DOWN (host)
+  const int wc = sh.col_j[nc - 1] + 2 - kfirst + 1;  // <= the form's window (host)
   const int wr = sh.row_i[nr - 1] + 2 - in_base + 1; // <= RS_MAX_IN (host)
   const int esz = elem_bytes<TIn>(a.in_dtype);
   for (int r = tid; r < wr; r += RS_THREADS)
     sh.in_off[r] = (int64_t)clamp_idx(in_base + r, n) * a.in_sh * esz;
-  if (UP) {
+  if (FORM == RS_CELLS) {
     for (int c = tid; c < nc; c += RS_THREADS)
       if (c == 0 || sh.col_j[c] != sh.col_j[c - 1]) sh.start[sh.col_j[c] - 1 - kfirst] = c;
     if (tid == 0) sh.start[wc - 3] = nc;
@@ -525,7 +523,7 @@ __global__ void __launch_bounds__(RS_THREADS, 3)
   char* out = static_cast<char*>(a.out) +
               (plane * a.out_sc + (int64_t)(r0 + q0) * a.out_sh + (int64_t)c0 * a.out_sw) * osz;
   const int64_t row_bytes = a.out_sh * osz;
-  if constexpr (UP) {
+  if constexpr (FORM == RS_CELLS) {
     const int cells = wc - 3;
     int most = 0;  // outputs of the fullest cell
     for (int k = lane; k < cells; k += 32) most = max(most, sh.start[k + 1] - sh.start[k]);
@@ -537,13 +535,13 @@ __global__ void __launch_bounds__(RS_THREADS, 3)
     else
       row_pass_up<BMODE, TOut, 4>(a, sh, warp, lane, nq, nc, cells, most, out, row_bytes, eps, beta);
   } else {
-    row_pass_down<BMODE, TOut>(a, sh, warp, lane, nq, nc, kfirst, out, row_bytes, eps, beta);
+    row_pass_outputs<BMODE, TOut>(a, sh, warp, lane, nq, nc, kfirst, out, row_bytes, eps, beta);
   }
 }
 
 template <int BMODE, class TIn, class TOut>
 cudaError_t launch_form(const ResampleArgs& a, float eps, float beta, cudaStream_t stream) {
-  if (!a.tiled) {
+  if (a.form == RS_DIRECT) {
     const dim3 block(32, 8);
     const dim3 grid((unsigned)((a.m_out + 31) / 32), (unsigned)((a.n_out + 7) / 8),
                     (unsigned)a.planes);
@@ -553,10 +551,12 @@ cudaError_t launch_form(const ResampleArgs& a, float eps, float beta, cudaStream
   const int tr = RS_WARPS * a.warp_rows;
   const dim3 grid((unsigned)((a.m_out + a.tile_cols - 1) / a.tile_cols),
                   (unsigned)((a.n_out + tr - 1) / tr), (unsigned)a.planes);
-  if (a.up)
-    resample_tiled_kernel<BMODE, TIn, TOut, true><<<grid, RS_THREADS, 0, stream>>>(a, eps, beta);
+  if (a.form == RS_CELLS)
+    resample_tiled_kernel<BMODE, TIn, TOut, RS_CELLS><<<grid, RS_THREADS, 0, stream>>>(a, eps, beta);
+  else if (a.form == RS_OUTPUTS)
+    resample_tiled_kernel<BMODE, TIn, TOut, RS_OUTPUTS><<<grid, RS_THREADS, 0, stream>>>(a, eps, beta);
   else
-    resample_tiled_kernel<BMODE, TIn, TOut, false><<<grid, RS_THREADS, 0, stream>>>(a, eps, beta);
+    resample_tiled_kernel<BMODE, TIn, TOut, RS_REDUCED><<<grid, RS_THREADS, 0, stream>>>(a, eps, beta);
   return cudaGetLastError();
 }
 
@@ -607,31 +607,13 @@ cudaError_t launch_resample(const ResampleArgs& a_in, float eps, float beta, int
   ResampleArgs a = a_in;
   a.div_y = axis_div(a.n, a.n_out);
   a.div_x = axis_div(a.m, a.m_out);
-  // spacing ratios (n - 1)/(n_out - 1) <= 2 per axis, and something to
-  // interpolate on both
-  a.tiled = a.n > 1 && a.m > 1 &&
-            (a.m_out == 1 || 2 * (a.m_out - 1) >= (a.m - 1)) &&
-            (a.n_out == 1 || 2 * (a.n_out - 1) >= (a.n - 1));
-  if (a.tiled) {
-    a.up = a.m_out >= a.m;
-    // magnified: as many columns as 64 window columns serve (a span of d input
-    // spacings touches at most ceil(d) + 4 samples), in whole words
-    int64_t tc = RS_TC_DOWN;
-    if (a.up) {
-      tc = (RS_WC_UP - 4) * (a.m_out - 1) / (a.m - 1) + 1;
-      tc = std::min<int64_t>(tc, RS_TC_MAX) & ~int64_t(3);
-    }
-    a.tile_cols = (int)tc;
-    // rows per warp: each warp loads 3 rows more than its cells, so more rows
-    // cost less, as long as about every SM gets a tile (reduced rows: three
-    // in four SMs; halving 4 rows there doubles the halo's share)
-    const int sms = resample_sms(), least = a.n_out >= a.n ? sms : 3 * sms / 4;
-    const int64_t strips = (a.m_out + tc - 1) / tc * a.planes;
-    int rows = a.n_out >= a.n && a.up ? RS_MAX_ROWS : RS_DOWN_ROWS;
-    while (rows > 1 && strips * ((a.n_out + RS_WARPS * rows - 1) / (RS_WARPS * rows)) < least)
-      rows >>= 1;
-    a.warp_rows = rows;
-  }
+  const RsPlan plan = rs_plan(
+      RsShape{a.n, a.m, a.planes, a.n_out, a.m_out,
+              a.out_dtype == DT_U8 ? 1 : (a.out_dtype == DT_F32 ? 4 : 2)},
+      resample_sms());
+  a.form = plan.form;
+  a.tile_cols = plan.cols;
+  a.warp_rows = plan.rows;
   const int i = a.in_dtype, o = a.out_dtype;
   if (i == DT_U8 && o == DT_U8) return launch_beta<uint8_t, uint8_t>(a, eps, beta, bmode, stream);
   if (i == DT_F16 && o == DT_F16) return launch_beta<__half, __half>(a, eps, beta, bmode, stream);

@@ -33,8 +33,7 @@ struct ResampleArgs {
   int out_vec4;                  // unit column stride, rows and planes of 4-element
                                  // multiples, 4-element aligned base
   // set by the launcher
-  int tiled;                     // the separable tiled kernel serves the ratios
-  int up;                        // the columns are magnified
+  int form;                      // how the call runs (RsForm of wd_resample_plan.h)
   int tile_cols;                 // output columns per tile
   int warp_rows;                 // output rows per warp
   AxisDiv div_y, div_x;          // division by n_out - 1, m_out - 1 (set by the launcher)
