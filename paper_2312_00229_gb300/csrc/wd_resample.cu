@@ -98,6 +98,11 @@ __device__ __forceinline__ float pos_h(float t) { return 0.5f * fmaf(t, t, -t); 
 // Cell index and offset of output index j on the endpoint-aligned grid of
 // n_out points over 0..n-1: i = floor(j (n-1) / (n_out-1)) exactly (by
 // multiply-high when the numerator fits 32 bits), t = remainder / (n_out-1).
+// WIDE: larger numerators (products of sides from 2^32 on) by a quotient in FP64,
+// at most one off as it is below 2^31, in place of a 64-bit integer division
+// (a line of 10^6 samples -> 3 10^6 57 -> 29 us; in the other kernels, which
+// find fewer positions, the longer code costs 1 to 2% at every size).
+template <bool WIDE = false>
 __device__ __forceinline__ void grid_pos(int j, int n, int n_out, const AxisDiv& d, int& i,
                                          float& t) {
   if (n <= 1 || n_out <= 1) { i = 0; t = 0.f; return; }
@@ -110,9 +115,23 @@ __device__ __forceinline__ void grid_pos(int j, int n, int n_out, const AxisDiv&
     t = (float)(int)(num - q * (uint32_t)den) * d.inv;
   } else {
     const int64_t num = (int64_t)j * (n - 1);
-    const int64_t q = num / den;
+    int64_t q, rest;
+    if (WIDE) {
+      q = (int64_t)((double)num * d.inv64);
+      rest = num - q * den;
+      if (rest < 0) {
+        --q;
+        rest += den;
+      } else if (rest >= den) {
+        ++q;
+        rest -= den;
+      }
+    } else {
+      q = num / den;
+      rest = num - q * den;
+    }
     i = (int)q;
-    t = (float)(num - q * den) * d.inv;
+    t = (float)rest * d.inv;
   }
   if (i > n - 2) { i = n - 2; t = 1.f; }  // last sample: t = 1 on the last cell
 }
@@ -152,7 +171,7 @@ __device__ __forceinline__ void rs_store(void* base, int64_t idx, float v, int d
 }
 
 // One thread per output, for reductions beyond 1/2 (little to share between
-// neighbouring outputs) and single-sample axes: all 16 loads are issued before the first is used,
+// neighbouring outputs): all 16 loads are issued before the first is used,
 // columns are interpolated in packed pairs.  1080p -> 480x270 uint8: 9.2 us with
 // run-time types and 64-bit positions, now 6.8.
 //
@@ -192,6 +211,23 @@ __device__ __forceinline__ float output_at(const ResampleArgs& a, int64_t plane,
   return u;
 }
 
+// The interpolant at cell i, offset t of a line of n samples `stride` apart.
+template <int BMODE, class TIn>
+__device__ __forceinline__ float line_at(const ResampleArgs& a, int64_t base, int64_t stride,
+                                         int i, int n, float t, float eps, float beta) {
+  if (n == 1) return rs_value<TIn>(rs_load_bits<TIn>(a.in, base, a.in_dtype), a.in_dtype);
+  uint32_t b[4];
+#pragma unroll
+  for (int p = 0; p < 4; ++p)
+    b[p] = rs_load_bits<TIn>(a.in, base + (int64_t)clamp_idx(i - 1 + p, n) * stride, a.in_dtype);
+  f2 v[4];
+#pragma unroll
+  for (int p = 0; p < 4; ++p) v[p] = pk_bc(rs_value<TIn>(b[p], a.in_dtype));
+  return eval2<BMODE>(cell2<BMODE>(v[0], v[1], v[2], v[3], eps, beta), pk_bc(t), pk_bc(pos_c0(t)),
+                      pk_bc(pos_h(t)))
+      .x;
+}
+
 template <int BMODE, class TIn, class TOut>
 __global__ void __launch_bounds__(256) resample_kernel(ResampleArgs a, float eps, float beta) {
   const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -206,6 +242,46 @@ __global__ void __launch_bounds__(256) resample_kernel(ResampleArgs a, float eps
   const float u = output_at<BMODE, TIn>(a, plane, i, ty, j, tx, eps, beta);
   rs_store<TOut>(a.out, plane * a.out_sc + r * a.out_sh + c * a.out_sw, u, a.out_dtype,
                  a.clamp_float);
+}
+
+// Single-sample axes, where one interpolant makes an output, and fewer rows than
+// a tile has warps, where most of a tile's warps would idle: one thread per
+// output column and `span` output rows, blockDim.y apart, or, of a single input
+// column, per output row and `span` columns, blockDim.x apart.  What the outputs of
+// a thread share is formed once: the column's position, and the output itself
+// where the input has one row or one column.
+template <int BMODE, class TIn, class TOut>
+__global__ void __launch_bounds__(256)
+    resample_lines_kernel(ResampleArgs a, float eps, float beta, int span) {
+  const int n = (int)a.n, m = (int)a.m;
+  const bool along_x = m == 1 && n > 1;
+  const int64_t c = (int64_t)blockIdx.x * blockDim.x * (along_x ? span : 1) + threadIdx.x;
+  int64_t r = (int64_t)blockIdx.y * blockDim.y * (along_x ? 1 : span) + threadIdx.y;
+  if (r >= a.n_out || c >= a.m_out) return;
+  const int64_t plane = blockIdx.z, base = plane * a.in_sc;
+  int64_t o = plane * a.out_sc + r * a.out_sh + c * a.out_sw;
+  const int64_t step = along_x ? blockDim.x * a.out_sw : blockDim.y * a.out_sh;
+  // outputs of this thread
+  const int64_t left = along_x ? (a.m_out - c - 1) / blockDim.x : (a.n_out - r - 1) / blockDim.y;
+  const int count = left < span ? (int)left + 1 : span;
+  int i, j;
+  float ty, tx;
+  if (along_x)
+    grid_pos<true>((int)r, n, (int)a.n_out, a.div_y, i, ty);
+  else
+    grid_pos<true>((int)c, m, (int)a.m_out, a.div_x, j, tx);
+  if (n == 1 || m == 1) {  // (uniform)
+    const float u = along_x ? line_at<BMODE, TIn>(a, base, a.in_sh, i, n, ty, eps, beta)
+                            : line_at<BMODE, TIn>(a, base, a.in_sw, j, m, tx, eps, beta);
+    for (int k = 0; k < count; ++k, o += step)
+      rs_store<TOut>(a.out, o, u, a.out_dtype, a.clamp_float);
+  } else {
+    for (int k = 0; k < count; ++k, o += step, r += blockDim.y) {
+      grid_pos<true>((int)r, n, (int)a.n_out, a.div_y, i, ty);
+      rs_store<TOut>(a.out, o, output_at<BMODE, TIn>(a, plane, i, ty, j, tx, eps, beta),
+                     a.out_dtype, a.clamp_float);
+    }
+  }
 }
 
 // ---- the tiled forms (sizes: wd_resample_plan.h) -------------------------------------
@@ -548,6 +624,16 @@ cudaError_t launch_form(const ResampleArgs& a, float eps, float beta, cudaStream
     resample_kernel<BMODE, TIn, TOut><<<grid, block, 0, stream>>>(a, eps, beta);
     return cudaGetLastError();
   }
+  if (a.form == RS_LINES) {
+    const bool along_x = a.m == 1 && a.n > 1;
+    const int64_t bx = a.tile_cols, by = 256 / bx, span = a.warp_rows;
+    const int64_t cols = bx * (along_x ? span : 1), rows = by * (along_x ? 1 : span);
+    const dim3 grid((unsigned)((a.m_out + cols - 1) / cols), (unsigned)((a.n_out + rows - 1) / rows),
+                    (unsigned)a.planes);
+    resample_lines_kernel<BMODE, TIn, TOut>
+        <<<grid, dim3((unsigned)bx, (unsigned)by), 0, stream>>>(a, eps, beta, (int)span);
+    return cudaGetLastError();
+  }
   const int tr = RS_WARPS * a.warp_rows;
   const dim3 grid((unsigned)((a.m_out + a.tile_cols - 1) / a.tile_cols),
                   (unsigned)((a.n_out + tr - 1) / tr), (unsigned)a.planes);
@@ -585,10 +671,11 @@ static int resample_sms() {
 }
 
 static AxisDiv axis_div(int64_t n, int64_t n_out) {
-  AxisDiv d{1u, 0, 0, 0, 0.f};
+  AxisDiv d{1u, 0, 0, 0, 0.f, 0.0};
   if (n <= 1 || n_out <= 1) return d;
   const uint64_t den = (uint64_t)(n_out - 1);
-  d.inv = (float)(1.0 / (double)den);
+  d.inv64 = 1.0 / (double)den;
+  d.inv = (float)d.inv64;
   // the largest numerator is (n_out - 1)(n - 1)
   if (den >= (1ull << 32) || (uint64_t)(n - 1) >= (1ull << 32) ||
       den * (uint64_t)(n - 1) >= (1ull << 32))

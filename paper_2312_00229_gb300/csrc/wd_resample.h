@@ -19,6 +19,7 @@ struct AxisDiv {
   int sh1, sh2;
   int fast;   // every numerator j (n - 1) of the axis is below 2^32
   float inv;  // 1 / d (for the cell offset t)
+  double inv64;  // 1 / d (for the quotient of larger numerators)
 };
 
 struct ResampleArgs {
@@ -34,8 +35,8 @@ struct ResampleArgs {
                                  // multiples, 4-element aligned base
   // set by the launcher
   int form;                      // how the call runs (RsForm of wd_resample_plan.h)
-  int tile_cols;                 // output columns per tile
-  int warp_rows;                 // output rows per warp
+  int tile_cols;                 // output columns per tile (RS_LINES: a block's)
+  int warp_rows;                 // output rows per warp (RS_LINES: outputs per thread)
   AxisDiv div_y, div_x;          // division by n_out - 1, m_out - 1 (set by the launcher)
 };
 

@@ -9,8 +9,9 @@
 
 namespace wdweno {
 
-// Three forms of the tiled kernel, and one thread per output (wd_resample.cu).
-enum RsForm { RS_REDUCED = 0, RS_CELLS = 1, RS_OUTPUTS = 2, RS_DIRECT = 3 };
+// Three forms of the tiled kernel, one thread per output, and one per line of
+// outputs (wd_resample.cu).
+enum RsForm { RS_REDUCED = 0, RS_CELLS = 1, RS_OUTPUTS = 2, RS_DIRECT = 3, RS_LINES = 4 };
 
 constexpr int RS_WARPS = 8;
 constexpr int RS_MAX_ROWS = 8;                 // output rows per warp, at most
@@ -32,8 +33,8 @@ struct RsShape {
 
 struct RsPlan {
   int form;
-  int cols;      // output columns of a tile
-  int rows;      // output rows per warp
+  int cols;      // output columns of a tile (RS_LINES: of a block)
+  int rows;      // output rows per warp (RS_LINES: outputs per thread)
   int64_t ctas;  // of the tiled kernel, with at least two rows per warp
 };
 
@@ -65,12 +66,26 @@ inline RsPlan rs_plan_tile(const RsShape& s, int form, int sms) {
   return RsPlan{form, (int)tc, rows, count(std::max(rows, 2))};
 }
 
+// Lines of outputs: a block's columns, and outputs per thread, more than one
+// once there are threads enough for every SM.
+inline RsPlan rs_plan_lines(const RsShape& s, int sms) {
+  const bool along_x = s.m == 1 && s.n > 1;
+  int cols = 1;
+  while (cols < (along_x ? 32 : 256) && cols < s.m_out) cols *= 2;
+  const int64_t by = 256 / cols;
+  const double outputs = double(s.m_out) * double(s.n_out) * double(s.planes);
+  int64_t span = std::max<int64_t>(1, int64_t(std::min(8.0, outputs / (1024.0 * sms))));
+  // (blocks along y fit the grid; along_x there are eight rows a block)
+  if (!along_x) span = std::max<int64_t>(span, (s.n_out + 65535 * by - 1) / (65535 * by));
+  return RsPlan{RS_LINES, cols, (int)span, 0};
+}
+
 inline RsPlan rs_plan(const RsShape& s, int sms) {
   const int64_t dx = s.m - 1, dx_out = s.m_out - 1, dy = s.n - 1, dy_out = s.n_out - 1;
-  // spacing ratios beyond 2 (little to share between neighbouring outputs), and
-  // nothing to interpolate on an axis
-  if ((dx_out > 0 && 2 * dx_out < dx) || (dy_out > 0 && 2 * dy_out < dy) || s.n == 1 || s.m == 1)
+  // spacing ratios beyond 2: little to share between neighbouring outputs
+  if ((dx_out > 0 && 2 * dx_out < dx) || (dy_out > 0 && 2 * dy_out < dy))
     return RsPlan{RS_DIRECT, 0, 0, 0};
+  if (s.n == 1 || s.m == 1 || s.n_out < RS_WARPS) return rs_plan_lines(s, sms);
   if (s.m_out < s.m) {
     // Reduced columns: 128 outputs with the window they need, or, where the rows
     // are magnified or the columns reduced by less than 1.12, the outputs of 128

@@ -15,8 +15,8 @@ pytestmark = pytest.mark.gpu
 TOL = 1e-5  # one resampling of O(1) values in FP32
 
 # far magnified (by outputs), reduced columns with magnified rows, about the same
-# spacing, single-sample axes and few rows: tiles of 128 outputs, warps of 8 rows, and
-# one more or less of each
+# spacing, single-sample axes and few rows (lines): tiles of 128 outputs, blocks
+# of 32 and 256 columns and of 8 rows, and one more or less of each
 SIZES = [(3, 3, 70, 400), (2, 2, 9, 1000), (9, 8, 64, 129), (20, 33, 161, 1100), (12, 40, 300, 640),
          (40, 300, 130, 160), (33, 257, 200, 129), (16, 131, 40, 128), (64, 130, 64, 131),
          (70, 200, 71, 190), (130, 135, 129, 134), (1, 40, 17, 257), (1, 9, 9, 31), (40, 1, 129, 33),
@@ -76,9 +76,9 @@ def test_row_interpolants_are_the_forms_own(dtype, beta, m, ow):
     line = torch.rand((2, 1, m), generator=g, device="cuda")
     line = (line * 255).to(dtype) if dtype == torch.uint8 else line
     p = api.Params(beta=beta)
-    want = api.resample(line, 1, ow, p)
+    want = api.resample(line, 1, ow, p)  # lines
     assert torch.equal(api.resample(line, 9, ow, p), want.expand(2, 9, ow).contiguous())
-    for n, oh in ((40, 40), (40, 70), (40, 25), (40, 9), (5, 7)):  # tiles, direct
+    for n, oh in ((40, 40), (40, 70), (40, 25), (40, 9), (5, 7)):  # tiles, direct, lines
         y = api.resample(line.expand(2, n, m).contiguous(), oh, ow, p)
         assert torch.equal(y, want.expand(2, oh, ow)), (n, oh)
 
@@ -92,7 +92,7 @@ def test_column_interpolants_are_the_forms_own(dtype, beta, n, oh):
     line = torch.rand((2, n, 1), generator=g, device="cuda")
     line = (line * 255).to(dtype) if dtype == torch.uint8 else line
     p = api.Params(beta=beta)
-    want = api.resample(line, oh, 1, p)
+    want = api.resample(line, oh, 1, p)  # lines
     assert torch.equal(api.resample(line, oh, 300, p), want.expand(2, oh, 300).contiguous())
     for m, ow in ((40, 40), (40, 100), (40, 1000), (40, 38), (40, 25), (40, 9)):  # tiles, direct
         y = api.resample(line.expand(2, n, m).contiguous(), oh, ow, p)

@@ -1,8 +1,9 @@
 """Every plan of a resampling call keeps the kernel's bounds (window columns,
 input rows and cells of a warp, grid), and the form follows the measured rule:
 by cells where a tile's cells have work for its lanes, by outputs where the
-columns are magnified so far that they have not.  The plan's header, compiled
-for the host."""
+columns are magnified so far that they have not, lines for single-sample axes
+and fewer rows than a tile has warps.  The plan's header, compiled for the
+host."""
 import os
 import random
 import shutil
@@ -13,7 +14,7 @@ import pytest
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
                     "paper_2312_00229_gb300", "csrc")
 SMS = 152
-REDUCED, CELLS, OUTPUTS, DIRECT = range(4)
+REDUCED, CELLS, OUTPUTS, DIRECT, LINES = range(5)
 
 SRC = r"""
 #include <cstdio>
@@ -82,6 +83,11 @@ def test_every_plan_keeps_the_kernels_bounds(plans):
         seen.add(form)
         if form == DIRECT:
             continue
+        if form == LINES:
+            assert cols in (1, 2, 4, 8, 16, 32, 64, 128, 256) and rows >= 1
+            per_block = 256 // cols * (1 if m == 1 and n > 1 else rows)
+            assert (no + per_block - 1) // per_block <= 65535
+            continue
         assert n > 1 and m > 1 and cols >= 4 and cols % 4 == 0
         assert cols <= (tc_max if form == CELLS else 128)
         assert rows in (1, 2, 4, 8) and (rows < 8 or (no >= n and form != REDUCED))
@@ -100,7 +106,7 @@ def test_every_plan_keeps_the_kernels_bounds(plans):
             assert _cell(r1, n, no) - _cell(r0, n, no) + 4 <= max_in
             for q in range(r0, r1 + 1, rows):
                 assert _cell(min(q + rows - 1, r1), n, no) - _cell(q, n, no) < max_cells
-    assert seen == {REDUCED, CELLS, OUTPUTS, DIRECT}
+    assert seen == {REDUCED, CELLS, OUTPUTS, DIRECT, LINES}
 
 
 @pytest.mark.parametrize("form,shapes", [
@@ -112,6 +118,8 @@ def test_every_plan_keeps_the_kernels_bounds(plans):
                (3, 540, 960, 600, 1000, 1), (3, 540, 960, 4320, 500, 1),
                (3, 222, 987, 206, 914, 2)]),
     (REDUCED, [(3, 4317, 7677, 3240, 5760, 1), (3, 2160, 3840, 1270, 2258, 1)]),
+    (LINES, [(1, 1, 1000, 1000, 3000, 1), (1, 400000, 1, 500000, 1, 1), (1, 1, 1, 1, 1, 4),
+             (1, 6, 900, 7, 2000, 1)]),
     (DIRECT, [(3, 1080, 1920, 270, 480, 1), (3, 300, 300, 100, 900, 4)])])
 def test_form_follows_the_rule(plans, form, shapes):
     assert [g[0] for g in plans(shapes)[1]] == [form] * len(shapes)
