@@ -110,7 +110,8 @@ __global__ void __launch_bounds__(SETUP_THREADS) batched_setup_kernel(BatchedArg
       const int n = (int)in.height;
 #pragma unroll
       for (int j = 0; j < CANDS; ++j) {
-        const int r0 = g_cands[j], b0 = (n - 1) / r0 + 1, r = (n - 1) / b0 + 1;
+        const int r0 = g_cands[j], b0 = (n - 1) / r0 + 1;
+        const int r = r0 < batched::EVEN_FROM ? min(r0, n) : (n - 1) / b0 + 1;  // (even_band)
         const float bands = float((n - 1) / r + 1);
         c[j].tiles += strips * bands;
         c[j].steps += strips * (float(n) + bands * TILE_FILL);
