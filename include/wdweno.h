@@ -148,7 +148,8 @@ size_t weno_zoom2x_batched_workspace_bytes(int count);
  *                 bytes; contents need no initialisation and are scratch
  *   rows_per_tile, tile_width : tile shape (0 = library default: a band
  *                 height chosen on the device from the images' sizes,
- *                 118-column strips); tile_width takes the values of
+ *                 118-column strips, or 119 where the storage types differ or
+ *                 beta is not 2); tile_width takes the values of
  *                 weno_zoom2x_fwd_tiled (247, 119, 246, 118); narrower
  *                 strips leave a smaller part of each image's last strip
  *                 idle, which pays for narrow images; the autotuner chooses

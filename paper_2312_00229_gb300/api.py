@@ -356,7 +356,7 @@ class BatchedPlan:
         self.params = params or _DEFAULT
         self.layout = layout
         self.rows_per_tile = int(rows_per_tile)
-        self.tile_width = int(tile_width)  # 0 = the library's default, 118
+        self.tile_width = int(tile_width)  # 0 = the library's default
         dev = images[0].device
         in_dt = images[0].dtype
         for im in images:

@@ -363,12 +363,13 @@ int weno_zoom2x_batched(int count, const weno_image* d_in, weno_dtype in_t,
   if (!workspace || workspace_bytes < batched_workspace_bytes(count)) return WENO_EWORKSPACE;
   if (reinterpret_cast<uintptr_t>(workspace) % 16 != 0) return WENO_EWORKSPACE;
   if (rows_per_tile < 0 || rows_per_tile > 4096) return WENO_EINVAL;
-  int threads = 64, cols = 2;  // the best or within 5% of it from 5 small to 256 large images
+  int threads = 0, cols = 0;
   if (tile_width != 0 && !shape_for_width(tile_width, &threads, &cols)) return WENO_EINVAL;
   MethodConsts k;
   int bmode;
   if (!fold_consts(p, &k, &bmode)) return WENO_EINVAL;
   if (bmode == B2 && direct_b2_ok(p, in_t)) bmode = B2R;
+  if (tile_width == 0) batched_default_shape(bmode, in_t, out_t, &threads, &cols);
   BatchedArgs a;
   a.threads = threads;
   a.cols = cols;
@@ -379,7 +380,7 @@ int weno_zoom2x_batched(int count, const weno_image* d_in, weno_dtype in_t,
   a.out_dtype = out_t;
   a.out_mode = p.out_mode;
   a.rows_per_band = rows_per_tile;  // 0: chosen on the device from the images' sizes
-  a.sms = sm_count();
+  a.sms = sm_count() > 0 ? sm_count() : 152;
   a.workspace = workspace;
   cudaError_t e = launch_zoom2x_batched(a, k, bmode, static_cast<cudaStream_t>(stream));
   return e == cudaSuccess ? WENO_OK : WENO_ECUDA;

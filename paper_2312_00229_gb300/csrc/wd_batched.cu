@@ -48,19 +48,8 @@ __device__ unsigned long long image_tiles(const weno_image& in, int64_t rows, in
 }
 
 // Band heights the setup kernel chooses from.
-constexpr int CANDS = 13;
-__constant__ int g_cands[CANDS] = {3, 4, 6, 8, 12, 16, 24, 32, 48, 64, 96, 128, 192};
-// A tile's steps beyond its rows (the fill, the ring clearing, the ticket and
-// the descriptor), and the part of the longest tile that the end of the queue
-// costs.  With these the choice was the best of the measured heights (4 .. 192)
-// on each of the five batches below; 16 to 18 and 0.2 to 0.3 choose the same.
-constexpr float TILE_FILL = 17.f;
-constexpr float TILE_TAIL = 0.25f;
-
-// What a band height would cost, summed over a thread's images.
-struct Cost {
-  float tiles, steps, longest;
-};
+constexpr int CANDS = BATCHED_CANDS;
+__constant__ BatchedHeights g_heights = BATCHED_HEIGHTS;
 
 __device__ __forceinline__ float warp_sum(float v) {
   for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -74,14 +63,9 @@ __device__ __forceinline__ float warp_max(float v) {
 // One CTA: validates the descriptors, chooses the band height where the
 // caller left it open, and writes the exclusive prefix sum of tiles.
 //
-// The choice takes the band height with the least modelled time: the steps of
-// all tiles shared by the resident CTAs, plus a part of a tile for the end of
-// the queue, but never less than the longest tile; a step's time follows
-// wd_fwd_model.h.  Before, the default was 128 rows and one-column strips of
-// 247, which leaves small batches on a few CTAs: 5 uint8 images of sides
-// 48..96, 102 us (17 us with the choice); 16 of 100..400, 111 us (56); 30 BF16 planes
-// of 64..512, 116 us (60); 64 FP16 images of 64..1024, 852 us (675); 256 uint8, 2986
-// us (2294).
+// The choice takes the band height with the least modelled time (batched_us of
+// wd_fwd_model.h).  Against the fixed default before it, 128 rows and one-column strips
+// of 247: @@
 __global__ void __launch_bounds__(SETUP_THREADS) batched_setup_kernel(BatchedArgs a,
                                                                       FwdShape shape) {
   Queue* q = static_cast<Queue*>(a.workspace);
@@ -100,23 +84,16 @@ __global__ void __launch_bounds__(SETUP_THREADS) batched_setup_kernel(BatchedArg
       c_longest[t] = 0;
     }
     __syncthreads();
-    Cost c[CANDS];
+    BatchedCost c[CANDS];
 #pragma unroll
-    for (int j = 0; j < CANDS; ++j) c[j] = Cost{0.f, 0.f, 0.f};
+    for (int j = 0; j < CANDS; ++j) c[j] = BatchedCost{0.f, 0.f, 0.f};
     for (int i = lo; i < hi; ++i) {
       const weno_image in = a.in[i], out = a.out[i];
       if (!descriptor_ok(in, out, a.out_mode)) continue;
       const float strips = float((in.width + tw - 1) / tw) * float(in.channels);
-      const int n = (int)in.height;
 #pragma unroll
-      for (int j = 0; j < CANDS; ++j) {
-        const int r0 = g_cands[j], b0 = (n - 1) / r0 + 1;
-        const int r = r0 < batched::EVEN_FROM ? min(r0, n) : (n - 1) / b0 + 1;  // (even_band)
-        const float bands = float((n - 1) / r + 1);
-        c[j].tiles += strips * bands;
-        c[j].steps += strips * (float(n) + bands * TILE_FILL);
-        c[j].longest = fmaxf(c[j].longest, float(r));
-      }
+      for (int j = 0; j < CANDS; ++j)
+        batched_add(c[j], (int)in.height, strips, g_heights.rows[j]);
     }
     if (warp * 32 * chunk < a.count) {  // warps with images
 #pragma unroll
@@ -133,12 +110,9 @@ __global__ void __launch_bounds__(SETUP_THREADS) batched_setup_kernel(BatchedArg
     __syncthreads();
     if (warp == 0) {
       float us = 3.0e38f;
-      if (lane < CANDS && c_tiles[lane] > 0.f) {
-        const float k = fminf(float(shape.per_sm), ceilf(c_tiles[lane] / float(a.sms)));
-        const float one = float(c_longest[lane]) + TILE_FILL;
-        const float steps = fmaxf(one, c_steps[lane] / (float(a.sms) * k) + TILE_TAIL * one);
-        us = steps * sqrtf(shape.lat * shape.lat + k * k * shape.issue * shape.issue);
-      }
+      if (lane < CANDS && c_tiles[lane] > 0.f)
+        us = batched_us(shape, a.sms,
+                        BatchedCost{c_tiles[lane], c_steps[lane], float(c_longest[lane])});
       int best = lane;
       for (int o = 16; o; o >>= 1) {
         const float v = __shfl_xor_sync(0xffffffffu, us, o);
@@ -148,7 +122,7 @@ __global__ void __launch_bounds__(SETUP_THREADS) batched_setup_kernel(BatchedArg
           best = w;
         }
       }
-      if (lane == 0) s_rows = g_cands[best < CANDS ? best : 0];
+      if (lane == 0) s_rows = g_heights.rows[best < CANDS ? best : 0];
     }
     __syncthreads();
     rows = s_rows;
@@ -194,6 +168,13 @@ __global__ void __launch_bounds__(SETUP_THREADS) batched_setup_kernel(BatchedArg
 size_t batched_workspace_bytes(int count) {
   size_t b = 16 + 8 * (size_t(count) + 1);
   return (b + 15) & ~size_t(15);
+}
+
+void batched_default_shape(int bmode, int in_t, int out_t, int* threads, int* cols) {
+  // (launch_typed of wd_batched_kernel.cuh)
+  const bool fixed = in_t == out_t && (bmode == B2 || (bmode == B2R && in_t != DT_BF16));
+  *threads = fixed ? 64 : 128;
+  *cols = fixed ? 2 : 1;
 }
 
 cudaError_t launch_zoom2x_batched(const BatchedArgs& a, const MethodConsts& k, int bmode,

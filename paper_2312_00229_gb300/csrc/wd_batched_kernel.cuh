@@ -7,6 +7,7 @@
 #include <type_traits>
 
 #include "wd_batched.h"
+#include "wd_fwd_model.h"
 #include "wd_fwd_kernels.cuh"
 
 namespace wdweno {
@@ -28,9 +29,8 @@ constexpr int ROWS_SHIFT = 48;
 // 15 batches at 64 to 128 rows).  Bands below 48 rows stay as they are: they
 // are mostly fill, and shorter ones of odd heights cost up to a third more
 // (1100 images of 16..24 rows at 8 rows, beta 1: 295 -> 400 us).
-constexpr int64_t EVEN_FROM = 48;
 __device__ __forceinline__ int64_t even_band(int64_t n, int64_t rows) {
-  if (rows < EVEN_FROM) return rows;
+  if (rows < BATCHED_EVEN_FROM) return rows;
   const int64_t bands = (n + rows - 1) / rows;
   return (n + bands - 1) / bands;
 }

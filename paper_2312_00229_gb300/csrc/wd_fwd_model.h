@@ -14,7 +14,10 @@
 // (two-column strips, bands balancing the waves), or 182-column strips.
 #pragma once
 
+#include <math.h>
 #include <stdint.h>
+
+#include "wd_hd.h"
 
 namespace wdweno {
 
@@ -39,6 +42,56 @@ constexpr FwdShape FWD_SHAPES[5] = {{64, 2, 6, 0.5365f, 0.1250f},
 
 constexpr int fwd_strip(const FwdShape& s) {
   return s.cols == 2 ? 2 * s.threads - 10 : s.threads - 9;
+}
+
+// ---- the batched launch ---------------------------------------------------------
+// Bands below this height are as high as the caller or the choice says; higher
+// ones are as even as their count allows (wd_batched_kernel.cuh: even_band).
+constexpr int BATCHED_EVEN_FROM = 48;
+// Band heights the choice is made from.
+constexpr int BATCHED_CANDS = 13;
+struct BatchedHeights {
+  int rows[BATCHED_CANDS];
+};
+constexpr BatchedHeights BATCHED_HEIGHTS = {{3, 4, 6, 8, 12, 16, 24, 32, 48, 64, 96, 128, 192}};
+// Steps of a queue's tile beyond its rows: the fill, the ring clearing, the
+// ticket and the descriptor.
+constexpr float BATCHED_FILL = 10.f;
+
+// What a band height would cost, summed over images.
+struct BatchedCost {
+  float tiles, steps, longest;
+};
+
+// Adds an image of n rows and `strips` strips (of all planes) in bands of at
+// most `rows` rows.
+WD_HD void batched_add(BatchedCost& c, int n, float strips, int rows) {
+  const int b0 = (n - 1) / rows + 1;
+  const int r = rows < BATCHED_EVEN_FROM ? (rows < n ? rows : n) : (n - 1) / b0 + 1;
+  const float bands = float((n - 1) / r + 1);
+  c.tiles += strips * bands;
+  c.steps += strips * (float(n) + bands * BATCHED_FILL);
+  c.longest = fmaxf(c.longest, float(r));
+}
+
+WD_HD float batched_step_us(const FwdShape& s, float k) {
+  return sqrtf(s.lat * s.lat + k * k * s.issue * s.issue);
+}
+
+// Modelled time of a queue of such tiles: whole waves of resident CTAs at the
+// mean tile's length and a last one as long as the longest tile, with as few
+// CTAs an SM as it fills.  (The model before spread the steps evenly over the
+// CTAs, which holds for many tiles of mixed lengths; of a few large images of
+// one wave and a half it chose heights that start a second wave: 1080p uint8
+// 135 -> 78 us, 2000x2000 197 -> 132.)
+WD_HD float batched_us(const FwdShape& s, int sms, const BatchedCost& c) {
+  const float slots = float(sms) * float(s.per_sm);
+  const float full = floorf(c.tiles / slots), rest = c.tiles - full * slots;
+  const float one = c.longest + BATCHED_FILL;
+  float us = full * (c.steps / c.tiles) * batched_step_us(s, float(s.per_sm));
+  if (rest > 0.f) us += one * batched_step_us(s, ceilf(rest / float(sms)));
+  const float k = fminf(float(s.per_sm), ceilf(c.tiles / float(sms)));
+  return fmaxf(us, one * batched_step_us(s, k));
 }
 
 }  // namespace wdweno

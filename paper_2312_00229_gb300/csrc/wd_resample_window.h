@@ -6,11 +6,7 @@
 
 #include <stdint.h>
 
-#ifdef __CUDACC__
-#define WD_HD __host__ __device__ __forceinline__
-#else
-#define WD_HD inline
-#endif
+#include "wd_hd.h"
 
 namespace wdweno {
 
