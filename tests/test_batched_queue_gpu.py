@@ -1,6 +1,6 @@
-"""A batch of one image whose tiles all fit the GPU at once takes about the
-one-launch forward's time at the same tile shape: no CTA holds a second tile
-while others have none (that is half as much again)."""
+"""A batch of one image of about one wave of tiles takes about the one-launch
+forward's time at the same tile shape: no CTA holds a second tile while others
+have none."""
 import pytest
 import torch
 
@@ -30,13 +30,14 @@ def _best_us(fn, reps=40):
     return times[len(times) // 4]
 
 
-def test_one_wave_of_tiles_runs_as_one_wave():
-    x = torch.randint(0, 256, (3, 1080, 1920), device="cuda", dtype=torch.uint8)
-    plan = api.BatchedPlan([x], rows_per_tile=64, tile_width=118)  # 17 x 17 x 3 tiles
+# (measured over the forward: 1.05, 1.02, 1.05; with tickets drawn in advance 1.37,
+# up to 1.94, 1.36, on some runs less.  Half of the way.)
+@pytest.mark.parametrize("n,m,rows", [(2000, 2000, 96), (2000, 2000, 128), (1500, 1500, 64)])
+def test_one_wave_of_tiles_runs_as_one_wave(n, m, rows):
+    x = torch.randint(0, 256, (3, n, m), device="cuda", dtype=torch.uint8)
+    plan = api.BatchedPlan([x], rows_per_tile=rows, tile_width=118)
     out = torch.empty_like(plan.outputs[0])
     batched = _best_us(plan.run)
-    single = _best_us(lambda: api.zoom2x_fwd(x, rows_per_tile=64, tile_width=118, out=out))
+    single = _best_us(lambda: api.zoom2x_fwd(x, rows_per_tile=rows, tile_width=118, out=out))
     assert torch.equal(plan.outputs[0], out)
-    # measured: 70 and 62 us; 90 with tickets drawn in advance.  Half of the
-    # way, which leaves 17% for a noisy run
-    assert batched < 1.32 * single, (batched, single)
+    assert batched < 1.2 * single, (batched, single)
