@@ -2,8 +2,6 @@
 // planes, one CTA per tile.  The tile body is in wd_fwd_tile.cuh.  Storage
 // types are compile-time parameters for the common pairs (wd_fwd_typed*.cu);
 // any other pair, and beta = 0, goes through the run-time-typed kernels here.
-#include <cmath>
-
 #include "wd_cascade.h"
 #include "wd_fwd_kernels.cuh"
 #include "wd_fwd_model.h"
@@ -22,10 +20,6 @@ int threads_fwd() { return fwd_tile::THREADS; }
 
 namespace {
 
-double step_us(const FwdShape& s, int64_t k) {
-  return std::sqrt(double(s.lat) * s.lat + double(k) * k * s.issue * s.issue);
-}
-
 // A plan is a function of its key alone, so the last ones are remembered (per
 // thread, a direct-mapped table): finding one scans some hundred candidates,
 // about 10 us of host time.
@@ -43,36 +37,6 @@ struct PlanSlot {
   FwdPlan plan;
 };
 
-FwdPlan find_plan(const PlanKey& q) {
-  FwdPlan best{fwd_tile::THREADS, 1, q.rows > 0 ? q.rows : q.n};
-  double best_us = 1e300;
-  for (const FwdShape& s : FWD_SHAPES) {
-    if (q.threads != 0 && (s.threads != q.threads || s.cols != q.cols)) continue;
-    const int64_t base = (q.m + fwd_strip(s) - 1) / fwd_strip(s) * q.planes;
-    const int64_t slots = (int64_t)q.sms * s.per_sm;
-    const double full = step_us(s, s.per_sm);
-    int64_t last = -1;
-    for (int64_t bands = 1; bands <= q.n && bands <= 4096; ++bands) {
-      const int64_t rows = q.rows > 0 ? q.rows : (q.n + bands - 1) / bands;
-      if (rows == last) continue;
-      // bands below 16 rows only where they still find idle CTA slots
-      if (bands > 1 && (rows < 2 || (rows < 16 && base * bands > 2 * slots))) break;
-      last = rows;
-      const int64_t ctas = base * ((q.n + rows - 1) / rows);
-      const int64_t rest = ctas % slots;
-      double t = double(ctas / slots) * full;
-      if (rest) t += step_us(s, (rest + q.sms - 1) / q.sms);
-      t *= double(rows < q.n ? rows : q.n) + FWD_FILL;
-      if (t < best_us - 1e-9) {
-        best_us = t;
-        best = FwdPlan{s.threads, s.cols, rows};
-      }
-      if (q.rows > 0) break;
-    }
-  }
-  return best;
-}
-
 }  // namespace
 
 FwdPlan fwd_plan_for(int64_t n, int64_t m, int64_t planes, int sms, int threads, int cols,
@@ -81,7 +45,8 @@ FwdPlan fwd_plan_for(int64_t n, int64_t m, int64_t planes, int sms, int threads,
   static thread_local PlanSlot table[64];
   const uint64_t h = (uint64_t)(n * 1000003 + m * 10007 + planes * 101 + rows * 7 + threads + cols);
   PlanSlot& slot = table[(h ^ (h >> 17)) & 63];
-  if (!slot.used || !(slot.key == key)) slot = PlanSlot{true, key, find_plan(key)};
+  if (!slot.used || !(slot.key == key))
+    slot = PlanSlot{true, key, fwd_find_plan(n, m, planes, key.sms, threads, cols, rows)};
   return slot.plan;
 }
 

@@ -5,6 +5,7 @@
 #include <stdint.h>
 
 #include "wd_common.cuh"
+#include "wd_fwd_model.h"
 
 namespace wdweno {
 
@@ -32,17 +33,7 @@ __host__ __device__ inline void set_store_modes(FwdArgs& a, int64_t esz) {
                base % (uint64_t)(4 * esz) == 0;
 }
 
-// Tile shape of a one-launch forward: `threads` per CTA, `cols` coarse columns
-// per thread (1: 256 or 128 threads, 247 or 119 output columns per strip; 2:
-// 128, 96 or 64 threads, 246, 182 or 118) and coarse rows per band.
-struct FwdPlan {
-  int threads, cols;
-  int64_t rows;
-};
-
-// The plan with the least modelled time for `planes` planes of n x m samples
-// on a GPU of `sms` SMs; threads (with cols) and rows are taken as given where
-// they are not 0.
+// fwd_find_plan (wd_fwd_model.h), the last plans remembered.
 FwdPlan fwd_plan_for(int64_t n, int64_t m, int64_t planes, int sms, int threads, int cols,
                      int64_t rows);
 

@@ -27,8 +27,7 @@ struct FwdShape {
   float lat, issue;   // us
 };
 
-constexpr float FWD_FILL = 6.3f;    // steps
-constexpr float FWD_LAUNCH = 2.2f;  // us
+constexpr float FWD_FILL = 6.3f;  // steps
 
 // Strips of 118, 246, 182, 119 and 247 output columns.  (182 is the library's
 // own choice only: it covers 512 columns with 576 thread columns where 118 takes
@@ -42,6 +41,51 @@ constexpr FwdShape FWD_SHAPES[5] = {{64, 2, 6, 0.5365f, 0.1250f},
 
 constexpr int fwd_strip(const FwdShape& s) {
   return s.cols == 2 ? 2 * s.threads - 10 : s.threads - 9;
+}
+
+// Tile shape of a one-launch forward: `threads` per CTA, `cols` coarse columns
+// per thread (1: 256 or 128 threads, 247 or 119 output columns per strip; 2:
+// 128, 96 or 64 threads, 246, 182 or 118) and coarse rows per band.
+struct FwdPlan {
+  int threads, cols;
+  int64_t rows;
+};
+
+// The plan with the least modelled time for `planes` planes of n x m samples
+// on a GPU of `sms` SMs; threads (with cols) and rows are taken as given where
+// they are not 0.
+inline FwdPlan fwd_find_plan(int64_t n, int64_t m, int64_t planes, int sms, int threads, int cols,
+                             int64_t given_rows) {
+  const auto step_us = [](const FwdShape& s, int64_t k) {
+    return sqrt(double(s.lat) * s.lat + double(k) * k * s.issue * s.issue);
+  };
+  FwdPlan best{256, 1, given_rows > 0 ? given_rows : n};
+  double best_us = 1e300;
+  for (const FwdShape& s : FWD_SHAPES) {
+    if (threads != 0 && (s.threads != threads || s.cols != cols)) continue;
+    const int64_t base = (m + fwd_strip(s) - 1) / fwd_strip(s) * planes;
+    const int64_t slots = (int64_t)sms * s.per_sm;
+    const double full = step_us(s, s.per_sm);
+    int64_t last = -1;
+    for (int64_t bands = 1; bands <= n && bands <= 4096; ++bands) {
+      const int64_t rows = given_rows > 0 ? given_rows : (n + bands - 1) / bands;
+      if (rows == last) continue;
+      // bands below 16 rows only up to two waves of CTAs
+      if (bands > 1 && (rows < 2 || (rows < 16 && base * bands > 2 * slots))) break;
+      last = rows;
+      const int64_t ctas = base * ((n + rows - 1) / rows);
+      const int64_t rest = ctas % slots;
+      double t = double(ctas / slots) * full;
+      if (rest) t += step_us(s, (rest + sms - 1) / sms);
+      t *= double(rows < n ? rows : n) + FWD_FILL;
+      if (t < best_us - 1e-9) {
+        best_us = t;
+        best = FwdPlan{s.threads, s.cols, rows};
+      }
+      if (given_rows > 0) break;
+    }
+  }
+  return best;
 }
 
 // ---- the batched launch ---------------------------------------------------------
