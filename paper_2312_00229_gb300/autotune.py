@@ -10,7 +10,8 @@ modelled time for the image's size (one launch) or for all of a batch's.
 This module times candidate shapes
 on the current GPU with CUDA events and caches the fastest per size class in
 a JSON file, keyed by device name, storage types, layout and size class
-(planes and the image sides rounded up to powers of two).
+(planes and the image sides rounded up to powers of two; of a batch the image
+count, the largest sides and the mean size).
 
 ``api.zoom2x_fwd(..., rows_per_tile=None)`` consults the cache; a miss uses the
 library's own default.
@@ -31,7 +32,7 @@ CANDIDATES = (0, 16, 24, 32, 48, 64, 96, 128, 192)
 # output columns per CTA: one column per thread (256 and 128 threads) and
 # two columns per thread (128 and 64 threads)
 TILE_WIDTHS = (247, 119, 246, 118)
-BATCHED_TILE_WIDTHS = TILE_WIDTHS  # the persistent kernel runs either tile
+BATCHED_TILE_WIDTHS = TILE_WIDTHS  # the persistent kernel runs each of them
 
 _lock = threading.Lock()
 _cache: Optional[Dict[str, int]] = None

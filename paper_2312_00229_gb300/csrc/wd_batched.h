@@ -27,7 +27,8 @@ size_t batched_workspace_bytes(int count);
 // CTA shape where the caller leaves the strip width open: two-column strips of
 // 118 for the kernels with storage types fixed at compile time (the best or
 // within 3% of it over 25 batches), one-column strips of 119 for the others
-// (different types, beta != 2: 8 to 17% less time than 118).
+// (different types, beta != 2: mostly 5 to 20% less time than 118; images about
+// 64 wide 15 to 20% more).
 void batched_default_shape(int bmode, int in_t, int out_t, int* threads, int* cols);
 
 cudaError_t launch_zoom2x_batched(const BatchedArgs& a, const MethodConsts& k, int bmode,

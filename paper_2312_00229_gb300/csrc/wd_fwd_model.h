@@ -8,7 +8,7 @@
 // all of them when many do.  Fitted to 680 launches over 48x64 .. 2160x3840,
 // 1 and 3 planes, uint8 to FP32, bands of 3 to 192 rows (rms error 4.4%).
 // Bands short enough to fill the GPU in one wave pay on small images, where
-// the sweep is a serial chain: 3x48x64 uint8 14.0 -> 6.2 us (rows 16 -> 3),
+// the sweep is a serial chain: 3x48x64 uint8 14.0 -> 5.9 us (rows 16 -> 3),
 // 3x256x256 FP32 15.2 -> 9.2 us, 1x300x700 FP16 14.4 -> 8.3 us, 3x512x512
 // 17.9 -> 15.9 us; from 1024x1024 on the plans are those of the rule before
 // (two-column strips, bands balancing the waves), or 182-column strips.
@@ -126,8 +126,8 @@ WD_HD float batched_step_us(const FwdShape& s, float k) {
 // mean tile's length and a last one as long as the longest tile, with as few
 // CTAs an SM as it fills.  (The model before spread the steps evenly over the
 // CTAs, which holds for many tiles of mixed lengths; of a few large images of
-// one wave and a half it chose heights that start a second wave: 1080p uint8
-// 135 -> 78 us, 2000x2000 197 -> 132.)
+// one wave and a half it chose heights that start a second wave: 1500x1500
+// uint8 137 -> 102 us, 2000x2000 196 -> 129.)
 WD_HD float batched_us(const FwdShape& s, int sms, const BatchedCost& c) {
   const float slots = float(sms) * float(s.per_sm);
   const float full = floorf(c.tiles / slots), rest = c.tiles - full * slots;

@@ -1,7 +1,8 @@
-// Forward kernels with the storage types fixed at compile time and
-// beta = 1: the same-type pairs.  (The run-time-typed kernels of wd_fwd.cu
-// issue 503 instructions a px-ch, these 250 to 330: 1x1025x1025 FP32 at
-// beta = 1 on the 2n-1 grid, 35.0 -> 18.7 us with the tile plan of wd_fwd_model.h.)
+// Forward kernels with the storage types fixed at compile time and beta = 1: the
+// same-type pairs.
+// (The run-time-typed kernels of wd_fwd.cu issue 484 instructions a px-ch, these 353,
+// FP32, 118-column strips, bands of 16 rows: 1x1025x1025 on the 2n-1 grid 34.4 -> 19.4
+// us, and with the run-time-typed kernels' best strips, 119, 26.1.)
 #include "wd_fwd_kernels.cuh"
 
 namespace wdweno {

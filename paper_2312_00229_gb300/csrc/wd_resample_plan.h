@@ -44,8 +44,8 @@ struct RsPlan {
 // as long as about every SM gets a CTA (reduced rows: three in four SMs, as
 // halving 4 rows there doubles the halo's share).  Magnified rows go down to 2
 // while three CTAs an SM, the most that fit, still hold them all, which shortens
-// every CTA's chain: 200x300 -> 800x1200 9.5 -> 8.2 us, 100x1000 -> 800x8000
-// 14.0 -> 11.7.
+// every CTA's chain: 200x300 -> 800x1200 9.5 -> 8.3 us, 100x1000 -> 800x8000
+// 14.0 -> 11.8.
 inline RsPlan rs_plan_tile(const RsShape& s, int form, int sms) {
   int64_t tc = RS_TC_DOWN;
   if (form != RS_REDUCED && s.m_out > 1) {
@@ -90,19 +90,19 @@ inline RsPlan rs_plan(const RsShape& s, int sms) {
     // Reduced columns: 128 outputs with the window they need, or, where the rows
     // are magnified or the columns reduced by less than 1.12, the outputs of 128
     // window columns (eight rows a warp where they are magnified, and two column
-    // passes in place of three).  540x960 -> 1080x900 16.4 -> 11.5 us, 222x987 ->
-    // 206x914 8.1 -> 7.1; but 2160x3840 -> 1270x2258 47.6 against 54.4 the other way.
+    // passes in place of three).  540x960 -> 1080x900 16.2 -> 11.3 us, 222x987 ->
+    // 206x914 8.2 -> 6.8; but 2160x3840 -> 1270x2258 47.5 against 53.6 by outputs.
     const bool near = 100 * dx < 112 * dx_out;
     return rs_plan_tile(s, s.n_out >= s.n || near ? RS_OUTPUTS : RS_REDUCED, sms);
   }
   // A few rows of magnified columns: a tile is little work, so few tiles
-  // (8x200000 -> 8x300000 32 -> 20 us).
+  // (8x200000 -> 8x300000 33 -> 20 us).
   if (dx_out < 2 * dx && s.n_out <= 2 * RS_WARPS) return rs_plan_tile(s, RS_OUTPUTS, sms);
   const RsPlan c = rs_plan_tile(s, RS_CELLS, sms), o = rs_plan_tile(s, RS_OUTPUTS, sms);
   const int64_t c_strips = (s.m_out + c.cols - 1) / c.cols;
   const int64_t o_strips = (s.m_out + o.cols - 1) / o.cols;
   if (2 * dx_out < 5 * dx) {
-    // Magnified less than 2.5 times: by cells (540x960 -> 1080x1920 14.8 us, 19.2 by
+    // Magnified less than 2.5 times: by cells (540x960 -> 1080x1920 14.4 us, 18.8 by
     // outputs), but at about the same spacing 64 window columns serve no more
     // outputs, and tiles by outputs are twice as wide (540x960 -> 600x1000 10.7 ->
     // 8.2 us).
@@ -116,8 +116,8 @@ inline RsPlan rs_plan(const RsShape& s, int sms) {
   // CTAs an SM either costs more.  (Fitted to 3x to 64x of 8x8 to 1080x1920, three
   // types.)  A strip by cells is 480 outputs at most, so from 8x on it has fewer
   // and fewer cells for its 64 places: us by cells and by outputs, 540x960 uint8 4x
-  // 35 and 45, 8x 112 and 166, 12x 311 and 366, 16x 799 and 643; 64x64 8x 6.4 and 5.1,
-  // 16x 12.5 and 8.8, 64x 356 and 88; 3x3 -> 4000x4000 950 and 32.
+  // 35 and 43, 8x 112 and 159, 12x 311 and 349, 16x 800 and 614; 64x64 8x 6.3 and 4.9,
+  // 16x 12.5 and 8.6, 64x 356 and 85; 3x3 -> 4000x4000 949 and 30.
   const int64_t f = (2 * dx_out + dx) / (2 * dx);  // outputs per cell
   int64_t banks = 1;                               // gcd(words from cell to cell, 32)
   if (f * s.out_bytes % 4 == 0)
