@@ -83,6 +83,14 @@ def _require_cuda(t: torch.Tensor, name: str):
         raise TypeError(f"{name}: unsupported dtype {t.dtype}")
 
 
+def _require_samples(x: torch.Tensor):
+    """Refuses what a zoom refuses of its input: for chains of zooms, which
+    allocate the first level's output before that zoom sees the input."""
+    _require_cuda(x, "x")
+    if x.numel() == 0:
+        raise ValueError("empty input")
+
+
 def _planes(t: torch.Tensor, layout: str):
     """(height, width, channels, stride_c, stride_h, stride_w) of a tensor,
     folding a leading batch dimension into the channel count when the planes
@@ -127,11 +135,7 @@ def _level_out(x: torch.Tensor, params: Params, layout: str, dtype) -> torch.Ten
     with planar rows padded to a multiple of four elements.  Only the next
     level reads it, and rows that all start on a four-element boundary are
     written with one vector store per thread and fine row (odd widths of the
-    2n-1 grid otherwise take three).  What the zoom refuses is refused before
-    the allocation."""
-    _require_cuda(x, "x")
-    if x.numel() == 0:
-        raise ValueError("empty input")
+    2n-1 grid otherwise take three)."""
     dtype = dtype or x.dtype  # (as the zoom's own output: None keeps the input's)
     h, w = out_hw(x.shape[-2], x.shape[-1], params)
     if layout == "hwc" or w % 4 == 0:
@@ -274,6 +278,8 @@ def cascade_zoom(x: torch.Tensor, levels: int, params: Optional[Params] = None, 
                 B.weno_zoom2x_cascade(xi, _DT[x.dtype], oi, _DT[out.dtype], levels, pc, base,
                                       nbytes, _stream(x.device)))
         return out
+    if levels > 1:
+        _require_samples(x)
     bounds = _level_bounds(x, params, levels)
     cur = x
     for lvl in range(levels):
@@ -334,6 +340,8 @@ def zoom_to(x: torch.Tensor, out_h: int, out_w: int, params: Optional[Params] = 
     params = params or _DEFAULT
     n, m = _hw(x, layout)
     k = zoom_levels(n, m, out_h, out_w)
+    if k > 0:
+        _require_samples(x)
     bounds = _level_bounds(x, params, k)
     cur = x
     for lvl in range(k):

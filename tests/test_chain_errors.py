@@ -15,6 +15,11 @@ def test_host_tensors_are_refused(shape):
         api.cascade_zoom(x, 2, api.Params(out_mode=1))
 
 
+def test_no_level_is_no_zoom():
+    x = torch.zeros((1, 4, 6))
+    assert api.cascade_zoom(x, 0) is x
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("shape", [(1, 4, 0), (3, 0, 5), (4, 0)])
 def test_empty_images_are_refused(shape):
